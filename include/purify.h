@@ -79,7 +79,11 @@ extern "C" {
 #define PURIFY_SCHEME_LAST       9
 
 /* ---- arithmetic of the matrix products -------------------------------- */
-#define PURIFY_FP64    0  /* float64 FMA on the SIMT pipes                          */
+#define PURIFY_FP64    0  /* float64: products exact to 2^-57 of the row norms on the
+                             tensor cores (8 integer digit planes, 64-bit sums), or
+                             float64 FMA on the SIMT pipe for small n (< 128), n above
+                             32768, values the digits cannot hold (infinities, NaN,
+                             row scales beyond 2^+-400) and too little device memory  */
 #define PURIFY_MIXED   1  /* float64 values held as integer digit planes in bf16,
                              multiplied exactly on the tcgen05 tensor cores with
                              fp32 accumulation in tensor memory, recombined in
@@ -125,7 +129,7 @@ typedef struct purify_options {
                             the idle SMs and are added in a fixed order (default 1;
                             0 = whole tiles, the grouping the batch engine uses) */
     int refine_fp64;     /* MIXED: float64 McWeeny steps X <- 3X^2 - 2X^3 (two float64
-                            products each, on the GPU's float64 pipe) appended to the
+                            products each) appended to the
                             run, which set the final idempotency (0 = none, default;
                             at most 2); stats.trace and stats.idem_err_fro then
                             describe the last of them                              */

@@ -327,6 +327,27 @@ int make_pool_map(CUtensorMap* map, const __nv_bfloat16* pool, int slots, int np
     return r == CUDA_SUCCESS ? PURIFY_OK : PURIFY_ERR_CUDA;
 }
 
+}  // namespace
+
+// 3D map over the eight planes of a float64 operand (quad_index in
+// f64_digits.cu): dims {4 n_pad, n_pad, 2}, box {64, 128, 1}: one box row is
+// 128 bytes, a 16-wide k-chunk of four planes; 128-byte swizzle.
+int make_quad_map(CUtensorMap* map, const __nv_bfloat16* planes, int n_pad) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return PURIFY_ERR_UNSUPPORTED;
+    if (((uintptr_t)planes & 15) || n_pad % TILE) return PURIFY_ERR_INVALID_ARG;
+    cuuint64_t dims[3] = {(cuuint64_t)4 * n_pad, (cuuint64_t)n_pad, 2};
+    cuuint64_t strides[2] = {(cuuint64_t)n_pad * 8, (cuuint64_t)n_pad * n_pad * 8};
+    cuuint32_t box[3] = {64, (cuuint32_t)TILE, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)planes, dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? PURIFY_OK : PURIFY_ERR_CUDA;
+}
+
+namespace {
+
 df to_df(double x) {
     const float h = (float)x;
     return {h, (float)(x - (double)h)};

@@ -1,0 +1,741 @@
+// Float64 symmetric steps on the tcgen05 tensor cores.
+//
+// GB300's float64 pipe runs 2 FMAs per clock and SM (1.26 TFLOP/s on the
+// chip), so a float64 product there is bound by that pipe at any size.  Here
+// the product is taken on the bf16 tensor pipe (1.9 PFLOP/s measured) without
+// giving up float64 accuracy: the operands are cut into integer digits whose
+// products and sums are exact in the fp32 accumulators, and the sums are put
+// together in 64-bit integers (the error-free splitting of Ozaki, Ogita,
+// Oishi and Rump, Numer. Algorithms 59 (2012), with digits of 7 bits).
+//
+// Digits.  Row i of a symmetric operand has the exponent e_i with
+// ||x_i||_2 <= 2^e_i (and > 2^(e_i - 2)); x_ij = 2^(e_i - 8) sum_p d_p 2^(-7p)
+// with |d_0| <= 256 and |d_p| <= 64 for p = 1..7: 57 bits below 2^e_i, an
+// entry's error is at most 2^(e_i - 58).  Digit p is stored as the bf16 value
+// d_p 2^(-7p), exactly.
+//
+// Product.  P_ij = 2^(e_i + e_j - 16) sum_l 2^(-7l) L_l with the level sums
+// L_l = sum_{p + q = l} sum_k d_p(i, k) d_q(j, k), l = 0..8 (p, q <= 7): 43
+// digit pairs.  What is left out (levels >= 9 and the digits' own rounding) is
+// about 2^-58 of ||x_i|| ||x_j||, below the rounding of a chain of n float64
+// FMAs.  (Without level 8, 36 pairs, off-diagonal entries came out 2.5 times
+// further off than with FMAs at n = 4096.)  A level sum over at most 1024 columns stays below 2^24 for
+// l <= 4 whatever the digits are (Cauchy-Schwarz for the pairs with d_0, at
+// most 3 x 1024 x 2^12 for the others) and is then exact in fp32; level 5 may
+// exceed it by a sixteenth in the worst case, at 2^-51 of the leading term per
+// unit, and levels 6 to 8 need no exactness.  So an accumulator is emptied at
+// least every 1024 columns, as an integer: each segment adds its levels,
+// shifted into units of 2^(e_i + e_j - 60), to a 64-bit integer per element
+// (|P_ij| <= 2^(e_i + e_j): the sum fits).  Integer sums do not depend on
+// their order, so the k-range of a tile may be cut anywhere and the result is
+// the same on every run and for any grid.
+//
+// Work.  Eight 128 x 128 accumulators would need twice the 512 columns of
+// tensor memory, so a tile's range is done in two passes: levels 0..3 from
+// digits 0..3 (10 digit pairs), then levels 4..8 from all digits (33; levels 7
+// and 8 share an accumulator).
+// Whole waves of tiles go round-robin, so that the CTAs walk k together and
+// share panels in L2; the tiles of the last, partial wave are cut evenly over
+// the grid at stage boundaries (at n = 256, three tiles on 30 CTAs).
+//
+// Measured, one step (float64 FMA kernel -> here): n = 256 281 -> 39 us, n =
+// 1000 1064 -> 87 us, n = 4096 57 ms -> 2.0 ms, of which the product kernel is
+// 1.57 ms: 1.95 PFLOP/s of digit pairs, the measured bf16 burst rate.  Errors of
+// one step against extended precision at n = 4096: largest 2.2e-15 -> 7e-17,
+// rms 1.8e-17 -> 2.4e-18.
+//
+// A step is three launches: split (unless the operand's digits are still at
+// hand), product, finish.  An operand with an infinity, a NaN or a row scale
+// outside 2^+-400 sets flags[0]: the kernels of that step and of all later
+// ones leave at once, and the caller takes the run up again from that step
+// with the float64 FMA kernel, which carries such values as before.
+#include "f64_digits.h"
+
+#include <algorithm>
+
+#include "digits_kernel.cuh"
+
+namespace purify {
+
+using namespace dk;
+
+int make_quad_map(CUtensorMap* map, const __nv_bfloat16* planes, int n_pad);  // digits_tc.cu
+
+namespace {
+
+constexpr int kDigits = 8;
+constexpr int kStages = 3;
+constexpr int kStageBytes = 64 * 1024;
+constexpr int kBoxBytes = TILE * 128;  // 128 rows of four planes' 16-wide k-chunks
+constexpr int kThreads = 64 + 32 * 8;
+constexpr int kMaxRegs = 168;
+constexpr int kExpLimit = 400;
+// MMAs per stage, which also measure the work: a high stage is 32 columns of
+// levels 0..3, a low stage 16 columns of levels 4..8
+constexpr int kHiCost = 20, kLoCost = 33;
+constexpr int kRange32 = 32;  // 1024 columns between two emptyings, in 32-column chunks
+constexpr int kCost32 = kHiCost + 2 * kLoCost;
+constexpr int kRangeCost = kRange32 * kCost32;
+constexpr int kMinCost = 60;  // a CTA gets at least this much of the last wave (about 2 us of MMAs)
+constexpr int ERR_F64_WAIT = 32;
+constexpr int kSmemBytes = 1024 + kStages * kStageBytes + 256;
+constexpr int64_t kF64DigitsMinN = 128, kF64DigitsMaxN = 1 << 15;
+
+struct F64Product {
+    CUtensorMap map_a, map_b;
+    unsigned long long* T;
+    int* flags;
+    int tiles_per_row, tiles, whole;  // whole: full waves of tiles
+};
+
+// The segments of one CTA, the same sequence in every role: a tile, a pass and
+// a run of stages.
+struct Segment {
+    int ti, tj, lo, k0, count;  // k0 in 32- (high) or 16-column (low) chunks
+};
+
+struct Walk {
+    int T, nk32, whole, grid, tile_cost;
+    int w = -1, tile = 0, pos = 0, end = 0;
+    long long tb, te;
+    __device__ explicit Walk(const F64Product& L) {
+        T = L.tiles_per_row;
+        nk32 = T * 4;
+        whole = L.whole;
+        grid = gridDim.x;
+        tile_cost = nk32 * kCost32;
+        const long long total = (long long)(L.tiles - whole * grid) * tile_cost;
+        tb = total * blockIdx.x / grid;
+        te = total * (blockIdx.x + 1) / grid;
+    }
+    __device__ bool next(Segment& g) {
+        for (;;) {
+            if (pos >= end) {
+                ++w;
+                if (w < whole) {
+                    tile = blockIdx.x + w * grid;
+                    pos = 0;
+                    end = tile_cost;
+                } else {
+                    if (tb >= te) return false;
+                    const int q = (int)(tb / tile_cost);
+                    tile = whole * grid + q;
+                    pos = (int)(tb - (long long)q * tile_cost);
+                    end = (int)min((long long)tile_cost, pos + (te - tb));
+                    tb += end - pos;
+                }
+            }
+            // the stages that start inside [pos, end) of this range's pass
+            const int r = pos / kRangeCost, base = r * kRangeCost;
+            const int kr = min(kRange32, nk32 - r * kRange32);
+            const int hc = kHiCost * kr, off = pos - base;
+            const int e = min(end - base, kCost32 * kr);
+            int s0, s1;
+            if (off < hc) {
+                const int eh = min(e, hc);
+                s0 = (off + kHiCost - 1) / kHiCost;
+                s1 = (eh + kHiCost - 1) / kHiCost;
+                g.lo = 0;
+                g.k0 = r * kRange32 + s0;
+                pos = base + eh;
+            } else {
+                s0 = (off - hc + kLoCost - 1) / kLoCost;
+                s1 = (e - hc + kLoCost - 1) / kLoCost;
+                g.lo = 1;
+                g.k0 = 2 * r * kRange32 + s0;
+                pos = base + e;
+            }
+            if (s1 > s0) {
+                g.count = s1 - s0;
+                decode_banded(tile, T, g.ti, g.tj);
+                return true;
+            }
+        }
+    }
+};
+
+// Descriptor offset (16-byte units) of digit plane p inside an operand's
+// 16-column chunk: four planes side by side in a 128-byte row.
+__host__ __device__ constexpr int quad_off(int p) { return ((p >> 2) * kBoxBytes + (p & 3) * 32) >> 4; }
+
+// Stage layout: A at 0, B at 32 KB.  High: two 16-column chunks of planes
+// 0..3 each; low: one chunk of planes 0..3 and 4..7.
+__device__ __forceinline__ void issue_high(uint32_t tmem, uint64_t da, uint64_t db, uint32_t later) {
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+        for (int l = 0; l < 4; ++l)
+#pragma unroll
+            for (int p = 0; p <= l; ++p)
+                mma_bf16(tmem + (uint32_t)(l * TILE), da + (uint64_t)(kk * (kBoxBytes >> 4) + quad_off(p)),
+                         db + (uint64_t)(kk * (kBoxBytes >> 4) + quad_off(l - p)), IDESC,
+                         (kk > 0 || p > 0) ? 1u : later);
+}
+
+__device__ __forceinline__ void issue_low(uint32_t tmem, uint64_t da, uint64_t db, uint32_t later) {
+#pragma unroll
+    for (int l = 4; l < 8; ++l)
+#pragma unroll
+        for (int p = 0; p <= l; ++p)
+            mma_bf16(tmem + (uint32_t)((l - 4) * TILE), da + (uint64_t)quad_off(p), db + (uint64_t)quad_off(l - p),
+                     IDESC, p > 0 ? 1u : later);
+#pragma unroll
+    for (int p = 1; p < 8; ++p)
+        mma_bf16(tmem + (uint32_t)(3 * TILE), da + (uint64_t)quad_off(p), db + (uint64_t)quad_off(8 - p), IDESC, 1u);
+}
+
+// 8 columns of the four accumulators, 32 lanes each; tmem_wait32 orders the
+// registers' use after the loads.
+__device__ __forceinline__ void tmem_issue32(uint32_t taddr, uint32_t (&r)[32]) {
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(r[8 * a]), "=r"(r[8 * a + 1]), "=r"(r[8 * a + 2]), "=r"(r[8 * a + 3]),
+                       "=r"(r[8 * a + 4]), "=r"(r[8 * a + 5]), "=r"(r[8 * a + 6]), "=r"(r[8 * a + 7])
+                     : "r"(taddr + (uint32_t)(a * TILE)));
+}
+
+__device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                   "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
+                   "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28])
+                 :: "memory");
+    asm volatile("" : "+r"(r[29]), "+r"(r[30]), "+r"(r[31])::"memory");
+}
+
+// The four accumulators of one element as a 64-bit integer in units of
+// 2^-60, modulo 2^64: 32-bit halves (64-bit integer operations run on the
+// float64 pipe).
+__device__ __forceinline__ uint2 levels_high(float a0, float a1, float a2, float a3) {
+    const int l0 = __float2int_rn(a0), l1 = __float2int_rn(a1 * 128.f), l2 = __float2int_rn(a2 * 16384.f),
+              l3 = __float2int_rn(a3 * 2097152.f);
+    // (l0 << 44) + (l1 << 37) + (l2 << 30) + (l3 << 23)
+    const unsigned int x = (unsigned int)l2 << 30, y = (unsigned int)l3 << 23, lo = x + y;
+    const unsigned int hi = ((unsigned int)l0 << 12) + ((unsigned int)l1 << 5) + (unsigned int)(l2 >> 2) +
+                            (unsigned int)(l3 >> 9) + (lo < x ? 1u : 0u);
+    return make_uint2(lo, hi);
+}
+
+__device__ __forceinline__ uint2 levels_low(float a4, float a5, float a6, float a7) {
+    const int l4 = __float2int_rn(a4 * 268435456.f), l5 = __float2int_rn(a5 * 34359738368.f),
+              l6 = __float2int_rn(a6 * 4398046511104.f), l7 = __float2int_rn(a7 * 562949953421312.f);
+    // (l4 << 16) + (l5 << 9) + (l6 << 2) + round(l7 / 32)
+    const int z = (l6 << 2) + ((l7 + 16) >> 5);
+    const unsigned int x = (unsigned int)l4 << 16, y = (unsigned int)l5 << 9, s = x + y, lo = s + (unsigned int)z;
+    const unsigned int hi = (unsigned int)(l4 >> 16) + (unsigned int)(l5 >> 23) + (unsigned int)(z >> 31) +
+                            (s < x ? 1u : 0u) + (lo < s ? 1u : 0u);
+    return make_uint2(lo, hi);
+}
+
+__global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_constant__ F64Product L) {
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t* full_bar = (uint64_t*)(base + kStages * kStageBytes);
+    uint64_t* empty_bar = full_bar + kStages;
+    uint64_t* tmem_full = empty_bar + kStages;
+    uint64_t* tmem_empty = tmem_full + 1;
+    uint64_t* drain = tmem_full + 2;
+    uint32_t* tmem_slot = (uint32_t*)(drain + 1);
+    volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (L.flags[0]) return;  // (written by earlier kernels only: uniform over the grid)
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 2 * kStages; ++i) mbar_init(smem_u32(&full_bar[i]), 1);
+        mbar_init(smem_u32(tmem_full), 1);
+        mbar_init(smem_u32(tmem_empty), 8);
+        mbar_init(smem_u32(drain), 1);
+        *abort_flag = 0;
+        fence_barrier_init();
+    }
+    if (warp == 1) tmem_alloc(smem_u32(tmem_slot), 4 * TILE);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    Walk walk(L);
+    Segment g;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int it = 0;
+            bool ok = true;
+            while (ok && walk.next(g)) {
+                for (int c = 0; c < g.count; ++c, ++it) {
+                    const int st = it % kStages;
+                    if ((it >= kStages &&
+                         !mbar_wait_for(smem_u32(&empty_bar[st]), (uint32_t)(((it / kStages) & 1) ^ 1))) ||
+                        *abort_flag) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t fb = smem_u32(&full_bar[st]);
+                    const uint32_t sa = smem_u32(base + (size_t)st * kStageBytes);
+                    const uint32_t sb = sa + 2 * kBoxBytes;
+                    mbar_arrive_expect_tx(fb, (uint32_t)kStageBytes);
+                    // high: two chunks of planes 0..3; low: one chunk of each four
+                    const int x0 = (g.k0 + c) * (g.lo ? 64 : 128), x1 = g.lo ? x0 : x0 + 64;
+                    tma_load_3d(sa, &L.map_a, fb, x0, g.ti * TILE, 0);
+                    tma_load_3d(sb, &L.map_b, fb, x0, g.tj * TILE, 0);
+                    tma_load_3d(sa + kBoxBytes, &L.map_a, fb, x1, g.ti * TILE, g.lo);
+                    tma_load_3d(sb + kBoxBytes, &L.map_b, fb, x1, g.tj * TILE, g.lo);
+                }
+            }
+            if (!ok) {
+                atomicOr(L.flags + 1, ERR_F64_WAIT);
+                *abort_flag = 1;
+            }
+            // wait (bounded) for the copies still in flight
+            for (int k = (it > kStages ? it - kStages : 0); k < it; ++k)
+                mbar_wait_for(smem_u32(&full_bar[k % kStages]), (uint32_t)((k / kStages) & 1));
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint64_t desc_base = smem_desc(smem_u32(base));
+            int it = 0, lt = 0;
+            bool ok = true;
+            for (; ok && walk.next(g); ++lt) {
+                if (lt > 0 && !mbar_wait_for(smem_u32(tmem_empty), (uint32_t)((lt - 1) & 1))) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                for (int c = 0; c < g.count; ++c, ++it) {
+                    const int st = it % kStages;
+                    if (!mbar_wait_for(smem_u32(&full_bar[st]), (uint32_t)((it / kStages) & 1))) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint64_t da = desc_base + (uint64_t)((st * kStageBytes) >> 4);
+                    const uint64_t db = da + (uint64_t)((2 * kBoxBytes) >> 4);
+                    if (g.lo)
+                        issue_low(tmem, da, db, c > 0 ? 1u : 0u);
+                    else
+                        issue_high(tmem, da, db, c > 0 ? 1u : 0u);
+                    mma_commit(smem_u32(&empty_bar[st]));
+                }
+                if (ok) mma_commit(smem_u32(tmem_full));
+            }
+            if (!ok) {
+                atomicOr(L.flags + 1, ERR_F64_WAIT);
+                *abort_flag = 1;
+            }
+            mma_commit(smem_u32(drain));
+            mbar_wait_for(smem_u32(drain), 0);
+        }
+    } else {
+        // epilogue warps: lane quarter warp % 4, columns 0..63 or 64..127
+        const int quarter = warp & 3, col0 = ((warp - 2) >> 2) * 64;
+        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)col0;
+        for (int lt = 0; walk.next(g); ++lt) {
+            bool ready = mbar_wait_for(smem_u32(tmem_full), (uint32_t)(lt & 1));
+            if (!ready) {
+                atomicOr(L.flags + 1, ERR_F64_WAIT);
+                *abort_flag = 1;
+            }
+            ready = __all_sync(0xffffffffu, ready && !*abort_flag);  // tcgen05.ld is warp-collective
+            if (!ready) break;
+            tc_fence_after();
+            // column-major inside a tile: a warp adds 32 consecutive integers
+            unsigned long long* t = L.T + (size_t)(g.tj * (g.tj + 1) / 2 + g.ti) * (TILE * TILE) + quarter * 32 + lane +
+                                    col0 * TILE;
+            uint32_t r[2][32];
+            tmem_issue32(taddr, r[0]);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                uint32_t(&v)[32] = r[q & 1];
+                tmem_wait32(v);
+                if (q < 7) {
+                    tmem_issue32(taddr + (uint32_t)(8 * (q + 1)), r[(q + 1) & 1]);
+                } else {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0)
+                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(tmem_empty)) : "memory");
+                }
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const float a0 = __uint_as_float(v[c]), a1 = __uint_as_float(v[8 + c]),
+                                a2 = __uint_as_float(v[16 + c]), a3 = __uint_as_float(v[24 + c]);
+                    const uint2 u = g.lo ? levels_low(a0, a1, a2, a3) : levels_high(a0, a1, a2, a3);
+                    atomicAdd(t + (8 * q + c) * TILE, (unsigned long long)u.y << 32 | u.x);
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        tmem_dealloc(tmem, 4 * TILE);
+    }
+}
+
+// ---- split: float64 rows -> exponents and digit planes ------------------------
+
+// Element offset of (plane p, row i, column j): planes 4m..4m+3 side by side
+// in 16-column chunks, 128-byte rows.
+__device__ __forceinline__ size_t quad_index(int p, int i, int j, int n_pad) {
+    return (size_t)(p >> 2) * 4 * n_pad * n_pad + (size_t)i * 4 * n_pad + ((j >> 4) << 6) + ((p & 3) << 4) + (j & 15);
+}
+
+template <int TPR, typename V, typename Op>
+__device__ __forceinline__ V row_reduce(V v, Op op) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if constexpr (TPR > 32) {
+        __shared__ V part[TPR / 32];
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+        __syncthreads();
+        v = part[0];
+#pragma unroll
+        for (int w = 1; w < TPR / 32; ++w) v = op(v, part[w]);
+    }
+    return v;
+}
+
+// TPR threads per row (a warp for short rows, the block of 256 for long ones),
+// four consecutive columns each.  Bound by HBM (8 bytes read and 16 written
+// per element): a row is read three times, the second and third time from L1.
+// Integer arithmetic and float32 only.
+template <int TPR>
+__global__ void __launch_bounds__(256)
+f64_split_kernel(const double* __restrict__ X, int n, int n_pad, __nv_bfloat16* __restrict__ planes,
+                 int* __restrict__ exps, int* flags, int step) {
+    // (a block of this launch may set it: decide once per block)
+    if (__syncthreads_or(*(volatile int*)flags != 0)) return;
+    const int i = (int)blockIdx.x * (256 / TPR) + (int)threadIdx.x / TPR;  // < n_pad, a multiple of 128
+    const int t = threadIdx.x % TPR;
+    const double* row = X + (size_t)i * n;
+    const bool in = i < n, vec = (n & 1) == 0;
+    auto load4 = [&](int j0, double (&x)[4]) {
+        x[0] = x[1] = x[2] = x[3] = 0.0;
+        if (!in) return;
+        if (vec && j0 + 3 < n) {
+            const double2 u = *(const double2*)(row + j0), v = *(const double2*)(row + j0 + 2);
+            x[0] = u.x;
+            x[1] = u.y;
+            x[2] = v.x;
+            x[3] = v.y;
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (j0 + c < n) x[c] = row[j0 + c];
+        }
+    };
+    unsigned int top = 0;  // the largest high word: sign off, exponent and 20 leading bits
+    unsigned int low = 0;  // whether a low word is set where the high word is zero
+    for (int j0 = 4 * t; j0 < n; j0 += 4 * TPR) {
+        double x[4];
+        load4(j0, x);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            top = max(top, (unsigned int)__double2hiint(x[c]) & 0x7fffffffu);
+            low |= (unsigned int)__double2loint(x[c]);
+        }
+    }
+    top = row_reduce<TPR>(top, [](unsigned int a, unsigned int b) { return max(a, b); });
+    low = row_reduce<TPR>(low, [](unsigned int a, unsigned int b) { return a | b; });
+    const int emax = (int)(top >> 20);
+    // sum of squares relative to 2^(emax - 1023), from the high words
+    float ss = 0.f;
+    for (int j0 = 4 * t; j0 < n; j0 += 4 * TPR) {
+        double x[4];
+        load4(j0, x);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const unsigned int h = (unsigned int)__double2hiint(x[c]) & 0x7fffffffu;
+            const int d = (int)(h >> 20) - emax;
+            const float m = d > -60 ? __uint_as_float((unsigned int)(127 + d) << 23 | (h & 0xfffffu) << 3) : 0.f;
+            ss = fmaf(m, m, ss);
+        }
+    }
+    ss = row_reduce<TPR>(ss, [](float a, float b) { return a + b; });
+    // the smallest k with 4^k > ss (raised by the truncation and the sum's rounding)
+    const int lg = (int)(__float_as_uint(ss * 1.01f) >> 23) - 127;
+    const int e = emax == 0 ? 0 : emax - 1023 + ((lg + 2) >> 1);
+    // outside the digits' range: not finite, denormal, or a scale beyond 2^+-400
+    const bool bad = emax == 0 ? (top | low) != 0 : (emax == 2047 || e > kExpLimit || e < -kExpLimit);
+    if (t == 0) {
+        exps[i] = e;
+        if (bad) atomicCAS(flags, 0, step + 1);
+    }
+    for (int j0 = 4 * t; j0 < n_pad; j0 += 4 * TPR) {
+        double x[4];
+        load4(j0, x);
+        uint32_t w[kDigits][2];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            // x 2^(57 - e), rounded to an integer of at most 58 bits
+            const unsigned int h = (unsigned int)__double2hiint(x[c]), l = (unsigned int)__double2loint(x[c]);
+            const int E = (int)((h >> 20) & 0x7ffu);
+            unsigned long long m = (unsigned long long)((h & 0xfffffu) | 0x100000u) << 32 | l;
+            const int sh = E - 1018 - e;  // <= 5
+            if (E == 0 || sh < -54)
+                m = 0;
+            else if (sh >= 0)
+                m <<= sh & 7;
+            else
+                m = (m + (1ull << (-sh - 1))) >> -sh;
+            long long f = (h >> 31) ? -(long long)m : (long long)m;
+            // balanced digits from the last one up: |d_p| <= 64
+            int d[kDigits];
+#pragma unroll
+            for (int p = kDigits - 1; p > 3; --p) {
+                f += 64;
+                d[p] = (int)((unsigned int)f & 127u) - 64;
+                f >>= 7;
+            }
+            int f32 = (int)f;
+#pragma unroll
+            for (int p = 3; p > 0; --p) {
+                f32 += 64;
+                d[p] = (f32 & 127) - 64;
+                f32 >>= 7;
+            }
+            d[0] = f32;
+            float scale = 1.f;
+#pragma unroll
+            for (int p = 0; p < kDigits; ++p) {
+                // d_p as a float by its bits (|d_p| <= 256), then its true scale; bf16 holds it exactly
+                const float v = (__int_as_float(0x4B400000 + d[p]) - 12582912.f) * scale;
+                const uint32_t b = __float_as_uint(v) >> 16;
+                if (c & 1)
+                    w[p][c >> 1] |= b << 16;
+                else
+                    w[p][c >> 1] = b;
+                scale *= 1.f / 128.f;
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < kDigits; ++p)
+            *(uint2*)(planes + quad_index(p, i, j0, n_pad)) = make_uint2(w[p][0], w[p][1]);
+    }
+}
+
+// ---- finish: fixed-point product -> the step's polynomial ----------------------
+
+__device__ __forceinline__ double warp_sum_d(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Y = cP P + cE E + cI I, C = dY Y + dI I (with mirror) over the 32 x 32 blocks
+// I <= J, and the reductions of step_f64_kernel.  Reads each fixed-point entry
+// once and clears it for the next step.
+__global__ void __launch_bounds__(256)
+f64_finish_kernel(unsigned long long* __restrict__ T, const int* __restrict__ ea, const int* __restrict__ eb,
+                  const double* __restrict__ E, double* __restrict__ C, int n, int blocks, double cP, double cE,
+                  double cI, double dY, double dI, double* red, const int* __restrict__ flags) {
+    __shared__ double tile[32][33];
+    __shared__ double rsum[3][8];
+    if (flags[0]) return;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    double s_tr = 0.0, s_idem = 0.0, s_fro = 0.0;
+    const bool affine = dY != 1.0 || dI != 0.0;
+    for (int b = blockIdx.x; b < blocks; b += gridDim.x) {
+        int J = (int)((sqrtf(8.f * (float)b + 1.f) - 1.f) * 0.5f);
+        while ((J + 1) * (J + 2) / 2 <= b) ++J;
+        while (J * (J + 1) / 2 > b) --J;
+        const int I = b - J * (J + 1) / 2;
+        unsigned long long* t = T + (size_t)((J >> 2) * ((J >> 2) + 1) / 2 + (I >> 2)) * (TILE * TILE) +
+                                (size_t)((J & 3) * 32) * TILE + (I & 3) * 32 + tx;
+        const int i = I * 32 + tx;
+        const int ei = ea[i];
+        unsigned long long v[4];
+        double e[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = ty + 8 * q, j = J * 32 + c;
+            v[q] = t[c * TILE];
+            t[c * TILE] = 0ull;
+            e[q] = (E && i < n && j < n) ? E[(size_t)j * n + i] : 0.0;
+        }
+        double sd = 0.0, sf = 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = ty + 8 * q, j = J * 32 + c;
+            double out = 0.0;
+            if (i < n && j < n && i <= j) {
+                const double p = (double)(long long)v[q] * __hiloint2double((ei + eb[j] - 60 + 1023) << 20, 0);
+                double y = cP * p + cE * e[q];
+                if (i == j) y += cI;
+                out = y;
+                if (affine) out = dY * y;
+                if (i == j) {
+                    out += dI;
+                    s_tr += y;
+                }
+                C[(size_t)j * n + i] = out;
+                if (red) {
+                    const double d = e[q] - p;
+                    double d2 = d, y2 = y;
+                    if (I == J && i != j) {  // (off-diagonal blocks are doubled below)
+                        d2 += d;
+                        y2 += y;
+                    }
+                    sd = fma(d2, d, sd);
+                    sf = fma(y2, y, sf);
+                }
+            }
+            tile[c][tx] = out;
+        }
+        const double wb = I == J ? 1.0 : 2.0;
+        s_idem += wb * sd;
+        s_fro += wb * sf;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = ty + 8 * q, i2 = I * 32 + r, j2 = J * 32 + tx;
+            if (i2 < n && j2 < n && i2 < j2) C[(size_t)i2 * n + j2] = tile[tx][r];
+        }
+        __syncthreads();
+    }
+    if (red) {
+        s_tr = warp_sum_d(s_tr);
+        s_idem = warp_sum_d(s_idem);
+        s_fro = warp_sum_d(s_fro);
+        if (tx == 0) {
+            rsum[0][ty] = s_tr;
+            rsum[1][ty] = s_idem;
+            rsum[2][ty] = s_fro;
+        }
+        __syncthreads();
+        if (threadIdx.x < 3) {
+            double v = 0.0;
+            for (int q = 0; q < 8; ++q) v += rsum[threadIdx.x][q];
+            atomicAdd(&red[threadIdx.x], v);
+        }
+    }
+}
+
+size_t plane_bytes(int n_pad) { return (size_t)n_pad * n_pad * kDigits * sizeof(__nv_bfloat16); }
+size_t t_bytes(int n_pad) {
+    return (size_t)upper_tiles(n_pad / TILE) * TILE * TILE * sizeof(unsigned long long);
+}
+
+int ensure_planes(F64Digits& f, int b) {
+    if (f.planes[b]) return PURIFY_OK;
+    PURIFY_CUDA_TRY(cudaMalloc(&f.planes[b], plane_bytes(f.cap_pad)));
+    PURIFY_CUDA_TRY(cudaMalloc(&f.exps[b], sizeof(int) * f.cap_pad));
+    return PURIFY_OK;
+}
+
+}  // namespace
+
+bool f64d_wanted(int64_t n) { return n >= kF64DigitsMinN && n <= kF64DigitsMaxN; }
+
+bool f64d_begin(F64Digits& f, int64_t n, int operands, cudaStream_t s, int* err) {
+    *err = PURIFY_OK;
+    if (!f64d_wanted(n)) return false;
+    const int n_pad = pad128(n);
+    auto ready = [&]() -> int {
+        if (n_pad > f.cap_pad) {
+            f64d_free(f);
+            int dev = 0;
+            PURIFY_CUDA_TRY(cudaGetDevice(&dev));
+            PURIFY_CUDA_TRY(cudaDeviceGetAttribute(&f.ctas, cudaDevAttrMultiProcessorCount, dev));
+            f.cap_pad = n_pad;
+            PURIFY_CUDA_TRY(cudaMalloc(&f.T, t_bytes(n_pad)));
+            PURIFY_CUDA_TRY(cudaMalloc(&f.flags, 2 * sizeof(int)));
+        }
+        f.n_pad = n_pad;
+        for (int b = 0; b < operands; ++b) PURIFY_TRY(ensure_planes(f, b));
+        PURIFY_CUDA_TRY(cudaFuncSetAttribute((const void*)f64_digit_product_kernel,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+        PURIFY_CUDA_TRY(cudaMemsetAsync(f.T, 0, t_bytes(n_pad), s));
+        PURIFY_CUDA_TRY(cudaMemsetAsync(f.flags, 0, 2 * sizeof(int), s));
+        return PURIFY_OK;
+    };
+    const int r = ready();
+    f.held[0] = f.held[1] = nullptr;
+    f.step = 0;
+    if (r == PURIFY_OK) return true;
+    f64d_free(f);
+    if (r == PURIFY_ERR_OOM)
+        cudaGetLastError();  // taken: the caller goes on without these buffers
+    else
+        *err = r;
+    return false;
+}
+
+static int split_into(F64Digits& f, int b, const double* X, int64_t n, cudaStream_t s) {
+    if (n <= 1024)
+        f64_split_kernel<32><<<f.n_pad / 8, 256, 0, s>>>(X, (int)n, f.n_pad, f.planes[b], f.exps[b], f.flags, f.step);
+    else
+        f64_split_kernel<256><<<f.n_pad, 256, 0, s>>>(X, (int)n, f.n_pad, f.planes[b], f.exps[b], f.flags, f.step);
+    PURIFY_CUDA_TRY(cudaGetLastError());
+    count_launches(1);
+    f.held[b] = X;
+    return PURIFY_OK;
+}
+
+int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, double* C, int64_t n, double cP,
+              double cE, double cI, double dY, double dI, double* red, cudaStream_t s) {
+    auto place = [&](const double* X, const double* other, int* b) -> int {
+        for (int q = 0; q < 2; ++q)
+            if (f.held[q] == X) {
+                *b = q;
+                return PURIFY_OK;
+            }
+        *b = (f.held[0] == other && other) ? 1 : 0;
+        return split_into(f, *b, X, n, s);
+    };
+    int a = 0, b = 0;
+    PURIFY_TRY(place(A, B, &a));
+    if (B == A)
+        b = a;
+    else
+        PURIFY_TRY(place(B, A, &b));
+    F64Product L;
+    PURIFY_TRY(make_quad_map(&L.map_a, f.planes[a], f.n_pad));
+    PURIFY_TRY(make_quad_map(&L.map_b, f.planes[b], f.n_pad));
+    L.T = f.T;
+    L.flags = f.flags;
+    L.tiles_per_row = f.n_pad / TILE;
+    L.tiles = (int)upper_tiles(L.tiles_per_row);
+    int grid = f.ctas;
+    L.whole = L.tiles / grid;
+    if (L.whole == 0) {
+        const long long cost = (long long)L.tiles * L.tiles_per_row * 4 * kCost32;
+        grid = (int)std::max<long long>(1, std::min<long long>(grid, cost / kMinCost));
+    }
+    f64_digit_product_kernel<<<grid, kThreads, kSmemBytes, s>>>(L);
+    const int64_t nb = (n + 31) / 32, blocks = nb * (nb + 1) / 2;
+    f64_finish_kernel<<<(unsigned)std::min<int64_t>(blocks, (int64_t)f.ctas * 8), 256, 0, s>>>(
+        f.T, f.exps[a], f.exps[b], E, C, (int)n, (int)blocks, cP, cE, cI, dY, dI, red, f.flags);
+    PURIFY_CUDA_TRY(cudaGetLastError());
+    count_launches(2);
+    for (int q = 0; q < 2; ++q)
+        if (f.held[q] == C) f.held[q] = nullptr;
+    ++f.step;
+    return PURIFY_OK;
+}
+
+int f64d_check(F64Digits& f, cudaStream_t s, int* redo_from) {
+    int v[2] = {0, 0};
+    *redo_from = -1;
+    PURIFY_CUDA_TRY(cudaMemcpyAsync(v, f.flags, sizeof(v), cudaMemcpyDeviceToHost, s));
+    PURIFY_CUDA_TRY(cudaStreamSynchronize(s));
+    if (v[1]) return PURIFY_ERR_DEVICE_TIMEOUT;
+    *redo_from = v[0] - 1;
+    return PURIFY_OK;
+}
+
+void f64d_free(F64Digits& f) {
+    for (int b = 0; b < 2; ++b) {
+        cudaFree(f.planes[b]);
+        cudaFree(f.exps[b]);
+    }
+    cudaFree(f.T);
+    cudaFree(f.flags);
+    f = F64Digits();
+}
+
+}  // namespace purify

@@ -1,0 +1,43 @@
+// Float64 steps on the tensor cores: exact digit products (f64_digits.cu).
+#pragma once
+
+#include <cuda_bf16.h>
+
+#include "internal.h"
+
+namespace purify {
+
+// Device buffers of a handle's float64 digit products (grow only, at most
+// 2^15 rows: 39 GB).  The digits of a step's operands are kept for the run's
+// next steps and forgotten at the next f64d_begin.
+struct F64Digits {
+    int n_pad = 0, cap_pad = 0, ctas = 0;
+    __nv_bfloat16* planes[2] = {nullptr, nullptr};
+    int* exps[2] = {nullptr, nullptr};  // row exponents of planes[b]
+    unsigned long long* T = nullptr;    // fixed-point product, upper 128 x 128 tiles; zero between steps
+    int* flags = nullptr;  // [0] the step (from 1) whose operand left the digits' range; [1] a wait that ran out
+    const double* held[2] = {nullptr, nullptr};  // the run's matrix whose digits planes[b] hold
+    int step = 0;                                // steps queued since f64d_begin
+};
+
+// Sizes that take the digit products (see f64_digits.cu).
+bool f64d_wanted(int64_t n);
+
+// Buffers for size n with the planes of `operands` (1 or 2) matrices, and a
+// cleared state for a new run's steps.  False when the size does not want
+// them or the device has no room (the caller then takes launch_step_f64); *err
+// receives other failures.
+bool f64d_begin(F64Digits& f, int64_t n, int operands, cudaStream_t s, int* err);
+
+// launch_step_f64 by exact digit products; A, B and E are exactly symmetric.
+int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, double* C, int64_t n, double cP,
+              double cE, double cI, double dY, double dI, double* red, cudaStream_t s);
+
+// Synchronises; the step (from 0) from which the run has to be taken up
+// again with launch_step_f64 because its operand cannot be held (-1: none;
+// that step and all later ones have written nothing).
+int f64d_check(F64Digits& f, cudaStream_t s, int* redo_from);
+
+void f64d_free(F64Digits& f);
+
+}  // namespace purify

@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "digits_tc.h"
+#include "f64_digits.h"
 #include "internal.h"
 #include "mixed.h"
 
@@ -355,6 +356,16 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
         release();
         return PURIFY_ERR_OOM;
     }
+    h->f64_on = false;
+    if (!mixed) {
+        const int r = begin_f64(h, 1);
+        if (r != PURIFY_OK) {
+            release();
+            return r;
+        }
+    }
+    bool digits = h->f64_on;  // float64 steps on the tensor cores
+    h->f64_on = false;
     int rc = PURIFY_ERR_NOT_CONVERGED;
     double homo = NAN, lumo = NAN;
     for (int i = 0; i < max_steps; ++i) {
@@ -389,7 +400,13 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
             r = launch_digit_step(st, s);
         } else {
             const double* Xi = Xf[(i + 1) & 1];
-            r = launch_step_f64(Xi, Xi, Xi, Xf[i & 1], n, cP, cE, 0.0, 1.0, 0.0, red, s);
+            if (digits) {
+                int redo = -1;
+                r = f64d_step(*h->f64, Xi, Xi, Xi, Xf[i & 1], n, cP, cE, 0.0, 1.0, 0.0, red, s);
+                if (r == PURIFY_OK) r = f64d_check(*h->f64, s, &redo);
+                if (r == PURIFY_OK && redo >= 0) digits = false;  // X_i does not fit in digits
+            }
+            if (!digits) r = launch_step_f64(Xi, Xi, Xi, Xf[i & 1], n, cP, cE, 0.0, 1.0, 0.0, red, s);
         }
         if (r != PURIFY_OK) {
             release();

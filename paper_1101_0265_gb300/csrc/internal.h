@@ -116,6 +116,7 @@ double pij_fixed_point(int i, int j);
 double pij_alpha(int i, int j, double c, double b, double bb);
 
 struct MixedState;
+struct F64Digits;
 
 }  // namespace purify
 
@@ -159,6 +160,8 @@ struct purify_ctx {
     std::vector<cudaEvent_t> pev;  // product timing events (pairs)
     int pev_used = 0;
     purify::MixedState* mixed = nullptr;
+    purify::F64Digits* f64 = nullptr;  // float64 products on the tensor cores (f64_digits.cu)
+    bool f64_on = false;               // the steps being queued take them
     // per-iteration reductions of the last run (purify_step_history)
     std::vector<double> hist_trace, hist_idem;
 };
@@ -185,6 +188,12 @@ int ensure_scratch(purify_ctx* h, int64_t doubles);
 // Make the dense F (and the density buffer X[0]) valid: from the CSR copy
 // when the Hamiltonian was loaded in block-sparse form.
 int ensure_dense_F(purify_ctx* h);
+// Start / end a run of float64 steps on the tensor cores (h->f64_on); `operands`
+// as for f64d_begin.  Where the size or the device's memory does not allow
+// them, f64_on stays false and the steps take the float64 FMA kernel.
+int begin_f64(purify_ctx* h, int operands);
+// Give the buffers of the float64 digit products back to the device.
+bool release_f64(purify_ctx* h);
 // The current F as CSR (csr_valid) for the bounds and the block-sparse split.
 inline CsrF csr_of(const purify_ctx* h) {
     CsrF c;

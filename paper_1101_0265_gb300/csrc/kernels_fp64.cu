@@ -1,6 +1,8 @@
 // Float64 SIMT kernels: the symmetric product of one purification step with
 // its fused polynomial epilogue (Eq. 1 with the f_i of Algorithm 1 and
-// Algorithm 2), the affine start f_0, and small helpers.
+// Algorithm 2), the affine start f_0, and small helpers.  Runs take this
+// product for n < 128 and where f64_digits.cu does not apply; the kernel-level
+// entry points take it always (they allocate nothing).
 //
 // GB300's float64 rate is about 1.1 TFLOP/s for the whole chip (roughly two
 // float64 FMAs per clock per SM), so this path is bound by the FMA pipe, not

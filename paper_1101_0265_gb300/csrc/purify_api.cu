@@ -5,6 +5,7 @@
 // Host arithmetic here is compiled without FMA contraction so that the
 // scalar schedule (alpha, beta, beta-bar, the branch test) is evaluated in
 // the plain float64 order the algorithms state.
+#include "f64_digits.h"
 #include "internal.h"
 #include "mixed.h"
 
@@ -362,9 +363,26 @@ static void free_buffers(purify_ctx* h) {
     h->p3_cap = 0;
 }
 
+int purify::begin_f64(purify_ctx* h, int operands) {
+    h->f64_on = false;
+    if (!f64d_wanted(h->n)) return PURIFY_OK;
+    if (!h->f64) h->f64 = new (std::nothrow) F64Digits();
+    if (!h->f64) return PURIFY_ERR_OOM;
+    int err = PURIFY_OK;
+    h->f64_on = f64d_begin(*h->f64, h->n, operands, h->stream, &err);
+    return err;
+}
+
+bool purify::release_f64(purify_ctx* h) {
+    if (!h->f64 || !h->f64->cap_pad) return false;
+    f64d_free(*h->f64);
+    return true;
+}
+
 static int ensure_capacity(purify_ctx* h, int64_t n) {
     if (n <= h->cap) return PURIFY_OK;
     free_buffers(h);
+    release_f64(h);
     const size_t bytes = sizeof(double) * (size_t)n * (size_t)n;
     PURIFY_CUDA_TRY(cudaMalloc(&h->F, bytes));
     PURIFY_CUDA_TRY(cudaMalloc(&h->X[0], bytes));
@@ -558,6 +576,8 @@ int purify_destroy(purify_t h) {
     cudaFree(h->csr_col);
     cudaFree(h->csr_val);
     mixed_free(h->mixed);
+    release_f64(h);
+    delete h->f64;
     for (cudaEvent_t e : h->pev) cudaEventDestroy(e);
     if (h->e0) cudaEventDestroy(h->e0);
     if (h->e1) cudaEventDestroy(h->e1);
@@ -726,6 +746,7 @@ int purify_set_hamiltonian_coo(purify_t h, int64_t n, int64_t nnz, const int64_t
         for (int I = 0; I < nb; ++I) h->f_pattern[(size_t)I * words + (I >> 6)] |= 1ull << (I & 63);
         for (int64_t i = 0; i < n; ++i) ptr[i + 1] += ptr[i];
         free_buffers(h);  // an earlier dense F and density
+        release_f64(h);
         if (h->csr_rows_cap < n + 1) {
             cudaFree(h->csr_ptr);
             h->csr_ptr = nullptr;
@@ -790,7 +811,11 @@ int purify_block_history(purify_t h, int* nnz_blocks, int cap, int* count) {
 static int step64(purify_ctx* h, const double* A, const double* B, const double* E, double* C,
                   double cP, double cE, double cI, double dY, double dI, int64_t slot) {
     PURIFY_TRY(product_begin(h));
-    PURIFY_TRY(launch_step_f64(A, B, E, C, h->n, cP, cE, cI, dY, dI, h->red + 4 * slot, h->stream));
+    double* red = h->red + 4 * slot;
+    if (h->f64_on)
+        PURIFY_TRY(f64d_step(*h->f64, A, B, E, C, h->n, cP, cE, cI, dY, dI, red, h->stream));
+    else
+        PURIFY_TRY(launch_step_f64(A, B, E, C, h->n, cP, cE, cI, dY, dI, red, h->stream));
     ++h->st.product_launches;
     return product_end(h);
 }
@@ -818,13 +843,31 @@ static int refine_f64(purify_ctx* h, int R) {
     PURIFY_TRY(ensure_red(h, 4 * (int64_t)(2 * R)));
     PURIFY_CUDA_TRY(cudaMemsetAsync(h->red, 0, sizeof(double) * 8 * R, h->stream));
     int x = h->cur;
-    for (int r = 0; r < R; ++r) {
-        double* X = h->X[x];
-        // S = X^2, reducing ||X - X^2||_F^2 (E = X)
-        PURIFY_TRY(step64(h, X, X, X, h->S, 1.0, 0.0, 0.0, 1.0, 0.0, 2 * r));
-        // X' = 3 S - 2 S X
-        PURIFY_TRY(step64(h, h->S, X, h->S, h->X[x ^ 1], -2.0, 3.0, 0.0, 1.0, 0.0, 2 * r + 1));
-        x ^= 1;
+    auto steps = [&](int r0) -> int {
+        for (int r = r0; r < R; ++r) {
+            double* X = h->X[x];
+            // S = X^2, reducing ||X - X^2||_F^2 (E = X)
+            PURIFY_TRY(step64(h, X, X, X, h->S, 1.0, 0.0, 0.0, 1.0, 0.0, 2 * r));
+            // X' = 3 S - 2 S X
+            PURIFY_TRY(step64(h, h->S, X, h->S, h->X[x ^ 1], -2.0, 3.0, 0.0, 1.0, 0.0, 2 * r + 1));
+            x ^= 1;
+        }
+        return PURIFY_OK;
+    };
+    PURIFY_TRY(begin_f64(h, 2));
+    const bool digits = h->f64_on;
+    int r = steps(0);
+    h->f64_on = false;
+    PURIFY_TRY(r);
+    if (digits) {
+        int redo = -1;
+        PURIFY_TRY(f64d_check(*h->f64, h->stream, &redo));
+        if (redo >= 0) {  // from the refinement step that could not be finished; its input is intact
+            const int r0 = redo / 2;
+            x = h->cur ^ (r0 & 1);
+            PURIFY_CUDA_TRY(cudaMemsetAsync(h->red + 8 * r0, 0, sizeof(double) * 8 * (R - r0), h->stream));
+            PURIFY_TRY(steps(r0));
+        }
     }
     h->cur = x;
     PURIFY_CUDA_TRY(cudaEventRecord(h->e1, h->stream));
@@ -838,12 +881,11 @@ static int refine_f64(purify_ctx* h, int R) {
     return PURIFY_OK;
 }
 
-static int run_fp64(purify_ctx* h, int scheme, double tol, int max_iter, double mu, Schedule& S,
-                    bool trace_rule, int* iters_out, std::vector<double>& red_host) {
-    PURIFY_TRY(ensure_work(h));
+static int run_fp64_steps(purify_ctx* h, int scheme, double tol, int max_iter, double mu, Schedule& S,
+                          bool trace_rule, int* iters_out, std::vector<double>& red_host) {
     const int64_t n = h->n;
     const double lmin = h->b.lmin, lmax = h->b.lmax;
-    int m = (int)S.alpha.size();
+    const int m = (int)S.alpha.size();
     if (is_fixed_mu(scheme) && (pmm_order(scheme) == 3 || is_asymmetric(scheme))) {
         // Higher-order and asymmetric P_{i,j}, scaled about c (1/2 when i = j):
         //   P_{3,3} = x^4 (35 - 84x + 70x^2 - 20x^3): V = 70 X_s - 20 X_s^2,
@@ -857,15 +899,6 @@ static int run_fp64(purify_ctx* h, int scheme, double tol, int max_iter, double 
         const double c = pi == pj ? 0.5 : pij_fixed_point(pi, pj);
         const double gamma = std::max((mu - lmin) / (1.0 - c), (lmax - mu) / c);
         const int ppi = products_per_iteration(scheme);
-        if (h->p3_cap < n) {
-            cudaFree(h->P3[0]);
-            cudaFree(h->P3[1]);
-            h->P3[0] = h->P3[1] = nullptr;
-            h->p3_cap = 0;
-            PURIFY_CUDA_TRY(cudaMalloc(&h->P3[0], sizeof(double) * (size_t)n * n));
-            PURIFY_CUDA_TRY(cudaMalloc(&h->P3[1], sizeof(double) * (size_t)n * n));
-            h->p3_cap = n;
-        }
         PURIFY_TRY(ensure_red(h, 4 * (int64_t)(ppi * m + 2)));
         PURIFY_CUDA_TRY(cudaMemsetAsync(h->red, 0, sizeof(double) * 4 * (ppi * m + 2), h->stream));
         PURIFY_CUDA_TRY(cudaEventRecord(h->e0, h->stream));
@@ -1022,6 +1055,42 @@ static int run_fp64(purify_ctx* h, int scheme, double tol, int max_iter, double 
     return PURIFY_OK;
 }
 
+// The float64 recursion: its products on the tensor cores (f64_digits.cu),
+// and, when an operand there cannot be held in digits (not finite, or a row
+// scale outside 2^+-400), the whole recursion again with the float64 FMA
+// kernel.  The buffers that either way needs come first.
+static int run_fp64(purify_ctx* h, int scheme, double tol, int max_iter, double mu, Schedule& S,
+                    bool trace_rule, int* iters_out, std::vector<double>& red_host) {
+    PURIFY_TRY(ensure_work(h));
+    const int64_t n = h->n;
+    const bool poly = is_fixed_mu(scheme) && (pmm_order(scheme) == 3 || is_asymmetric(scheme));
+    if (poly && h->p3_cap < n) {
+        cudaFree(h->P3[0]);
+        cudaFree(h->P3[1]);
+        h->P3[0] = h->P3[1] = nullptr;
+        h->p3_cap = 0;
+        PURIFY_CUDA_TRY(cudaMalloc(&h->P3[0], sizeof(double) * (size_t)n * n));
+        PURIFY_CUDA_TRY(cudaMalloc(&h->P3[1], sizeof(double) * (size_t)n * n));
+        h->p3_cap = n;
+    }
+    PURIFY_TRY(begin_f64(h, is_fixed_mu(scheme) ? 2 : 1));
+    if (h->f64_on) {
+        Schedule S1 = S;
+        const int r = run_fp64_steps(h, scheme, tol, max_iter, mu, S1, trace_rule, iters_out, red_host);
+        h->f64_on = false;
+        PURIFY_TRY(r);
+        int redo = -1;
+        PURIFY_TRY(f64d_check(*h->f64, h->stream, &redo));
+        if (redo < 0) {
+            S = S1;
+            return PURIFY_OK;
+        }
+        h->pev_used = 0;
+        h->st.product_launches = 0;
+    }
+    return run_fp64_steps(h, scheme, tol, max_iter, mu, S, trace_rule, iters_out, red_host);
+}
+
 int purify_run(purify_t h, int scheme, double tol, int max_iter) {
     if (!h) return PURIFY_ERR_INVALID_ARG;
     if (!h->have_F) return PURIFY_ERR_STATE;
@@ -1068,33 +1137,43 @@ int purify_run(purify_t h, int scheme, double tol, int max_iter) {
     const bool pooled_run = h->opt.precision == PURIFY_MIXED && h->opt.block_sparse && !trace_rule &&
                             pmm_order(scheme) != 3 && !is_asymmetric(scheme);
     if (!pooled_run) PURIFY_TRY(ensure_dense_F(h));
-    if (h->opt.precision == PURIFY_MIXED) {
-        if (trace_rule && h->opt.block_sparse) return PURIFY_ERR_UNSUPPORTED;
-        if (trace_rule) {
-            // the device-side schedule, unless the host one is asked for or
-            // the bounds already meet tol before the first step
-            const bool at_start = have_gap && std::max(S.beta0, 1.0 - S.betabar0) <= tol;
-            if (h->opt.host_schedule || at_start || max_iter == 0) {
-                r = run_mixed_trace(h, scheme, tol, max_iter, S, &h->cur, &iters);
+    auto dispatch = [&]() -> int {
+        int r;
+        if (h->opt.precision == PURIFY_MIXED) {
+            if (trace_rule && h->opt.block_sparse) return PURIFY_ERR_UNSUPPORTED;
+            if (trace_rule) {
+                // the device-side schedule, unless the host one is asked for or
+                // the bounds already meet tol before the first step
+                const bool at_start = have_gap && std::max(S.beta0, 1.0 - S.betabar0) <= tol;
+                if (h->opt.host_schedule || at_start || max_iter == 0) {
+                    r = run_mixed_trace(h, scheme, tol, max_iter, S, &h->cur, &iters);
+                } else {
+                    r = run_mixed_trace_graph(h, scheme, tol, max_iter, S, &h->cur, &iters);
+                    graph_run = true;
+                }
+            } else if (h->opt.block_sparse && (pmm_order(scheme) == 3 || is_asymmetric(scheme))) {
+                r = PURIFY_ERR_UNSUPPORTED;
+            } else if (pmm_order(scheme) == 3 || is_asymmetric(scheme)) {
+                r = run_mixed_poly(h, scheme, mu, S, &h->cur, red);
+            } else if (h->opt.block_sparse) {
+                r = run_block_sparse(h, scheme, S, &h->cur, red);
+                if (r == PURIFY_OK && h->mixed && !h->mixed->nnzb_history.empty())
+                    h->st.nnz_blocks = h->mixed->nnzb_history.back();
             } else {
-                r = run_mixed_trace_graph(h, scheme, tol, max_iter, S, &h->cur, &iters);
-                graph_run = true;
+                r = run_mixed(h, scheme, mu, S, &h->cur, red);
             }
-        } else if (h->opt.block_sparse && (pmm_order(scheme) == 3 || is_asymmetric(scheme))) {
-            r = PURIFY_ERR_UNSUPPORTED;
-        } else if (pmm_order(scheme) == 3 || is_asymmetric(scheme)) {
-            r = run_mixed_poly(h, scheme, mu, S, &h->cur, red);
-        } else if (h->opt.block_sparse) {
-            r = run_block_sparse(h, scheme, S, &h->cur, red);
-            if (r == PURIFY_OK && h->mixed && !h->mixed->nnzb_history.empty())
-                h->st.nnz_blocks = h->mixed->nnzb_history.back();
+            if (r == PURIFY_OK) r = refine_f64(h, h->opt.refine_fp64);
+            if (!trace_rule) iters = (int)S.alpha.size();
         } else {
-            r = run_mixed(h, scheme, mu, S, &h->cur, red);
+            r = run_fp64(h, scheme, tol, max_iter, mu, S, trace_rule, &iters, red);
         }
-        if (r == PURIFY_OK) r = refine_f64(h, h->opt.refine_fp64);
-        if (!trace_rule) iters = (int)S.alpha.size();
-    } else {
-        r = run_fp64(h, scheme, tol, max_iter, mu, S, trace_rule, &iters, red);
+        return r;
+    };
+    r = dispatch();
+    // the float64 products' buffers of an earlier run give way to this one's
+    if (r == PURIFY_ERR_OOM && release_f64(h)) {
+        cudaGetLastError();
+        r = dispatch();
     }
     if (r != PURIFY_OK) {
         h->st.status = r;
