@@ -36,11 +36,11 @@
 // and 8 share an accumulator).
 // Whole waves of tiles go round-robin, so that the CTAs walk k together and
 // share panels in L2; the tiles of the last, partial wave are cut evenly over
-// the grid at stage boundaries (at n = 256, three tiles on 30 CTAs).
+// the grid at stage boundaries (at n = 256, three tiles on 103 CTAs).
 //
-// Measured, one step (float64 FMA kernel -> here): n = 256 281 -> 39 us, n =
-// 1000 1064 -> 87 us, n = 4096 57 ms -> 2.0 ms, of which the product kernel is
-// 1.57 ms: 1.95 PFLOP/s of digit pairs, the measured bf16 burst rate.  Errors of
+// Measured, one step (float64 FMA kernel -> here): n = 256 281 -> 20.5 us, n =
+// 1000 1064 -> 64 us, n = 4096 57 ms -> 1.83 ms, of which the product kernel is
+// 1.56 ms: 1.95 PFLOP/s of digit pairs, the measured bf16 burst rate.  Errors of
 // one step against extended precision at n = 4096: largest 2.2e-15 -> 7e-17,
 // rms 1.8e-17 -> 2.4e-18.
 //
@@ -52,6 +52,7 @@
 #include "f64_digits.h"
 
 #include <algorithm>
+#include <type_traits>
 
 #include "digits_kernel.cuh"
 
@@ -76,7 +77,10 @@ constexpr int kHiCost = 20, kLoCost = 33;
 constexpr int kRange32 = 32;  // 1024 columns between two emptyings, in 32-column chunks
 constexpr int kCost32 = kHiCost + 2 * kLoCost;
 constexpr int kRangeCost = kRange32 * kCost32;
-constexpr int kMinCost = 60;  // a CTA gets at least this much of the last wave (about 2 us of MMAs)
+// A CTA gets at least this much of the last wave: one stage, so that in small
+// products no CTA empties its accumulators twice (n = 256, per step: 20.5 us with
+// 20, 24.6 with 30, 25.0 with 60; from n = 333 on the grid is full and it does not matter)
+constexpr int kMinCost = 20;
 constexpr int ERR_F64_WAIT = 32;
 constexpr int kSmemBytes = 1024 + kStages * kStageBytes + 256;
 constexpr int64_t kF64DigitsMinN = 128, kF64DigitsMaxN = 1 << 15;
@@ -87,6 +91,30 @@ struct F64Product {
     int* flags;
     int tiles_per_row, tiles, whole;  // whole: full waves of tiles
 };
+
+// Launched with programmatic stream serialization: the kernel's prologue runs
+// beside its predecessor's tail; memory is touched only after the
+// predecessor has completed, and the successor may then start its own prologue.
+__device__ __forceinline__ void grid_dependency_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_chained(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                           Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
 
 // The segments of one CTA, the same sequence in every role: a tile, a pass and
 // a run of stages.
@@ -207,23 +235,35 @@ __device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32]) {
 
 // The four accumulators of one element as a 64-bit integer in units of
 // 2^-60, modulo 2^64: 32-bit halves (64-bit integer operations run on the
-// float64 pipe).
+// float64 pipe).  Conversions of floats to integers run at 16 per clock and SM,
+// four per element would take 4096 cycles of an emptying; levels that stay below
+// 2^22 (0 and 1: |L_1| <= 2 x 2^8 x 64 x 32; 7 in units of 32) are read off the
+// bits of a sum with 1.5 2^23 instead, and one of the larger low levels in two
+// such pieces.
+constexpr float kMagic = 12582912.f;  // 1.5 2^23: bits 0x4B400000
+constexpr unsigned int kMagicBits = 0x4B400000u;
+
 __device__ __forceinline__ uint2 levels_high(float a0, float a1, float a2, float a3) {
-    const int l0 = __float2int_rn(a0), l1 = __float2int_rn(a1 * 128.f), l2 = __float2int_rn(a2 * 16384.f),
-              l3 = __float2int_rn(a3 * 2097152.f);
-    // (l0 << 44) + (l1 << 37) + (l2 << 30) + (l3 << 23)
-    const unsigned int x = (unsigned int)l2 << 30, y = (unsigned int)l3 << 23, lo = x + y;
-    const unsigned int hi = ((unsigned int)l0 << 12) + ((unsigned int)l1 << 5) + (unsigned int)(l2 >> 2) +
-                            (unsigned int)(l3 >> 9) + (lo < x ? 1u : 0u);
+    const unsigned int l0 = __float_as_uint(a0 + kMagic), l1 = __float_as_uint(fmaf(a1, 128.f, kMagic));
+    const int l2 = __float2int_rn(a2 * 16384.f), l3 = __float2int_rn(a3 * 2097152.f);
+    // (l0 << 44) + (l1 << 37) + (l2 << 30) + (l3 << 23); the magic bits shifted
+    // into the high half go off again
+    const unsigned int x = (unsigned int)l2 << 30, lo = x + ((unsigned int)l3 << 23);
+    const unsigned int hi = (l0 << 12) + (l1 << 5) + (unsigned int)(l2 >> 2) + (unsigned int)(l3 >> 9) +
+                            (lo < x ? 1u : 0u) - ((kMagicBits << 12) + (kMagicBits << 5));
     return make_uint2(lo, hi);
 }
 
 __device__ __forceinline__ uint2 levels_low(float a4, float a5, float a6, float a7) {
-    const int l4 = __float2int_rn(a4 * 268435456.f), l5 = __float2int_rn(a5 * 34359738368.f),
-              l6 = __float2int_rn(a6 * 4398046511104.f), l7 = __float2int_rn(a7 * 562949953421312.f);
-    // (l4 << 16) + (l5 << 9) + (l6 << 2) + round(l7 / 32)
-    const int z = (l6 << 2) + ((l7 + 16) >> 5);
-    const unsigned int x = (unsigned int)l4 << 16, y = (unsigned int)l5 << 9, s = x + y, lo = s + (unsigned int)z;
+    const int l4 = __float2int_rn(a4 * 268435456.f), l5 = __float2int_rn(a5 * 34359738368.f);
+    // level 6 = 4096 t + r, and level 7 (with 8) / 32
+    const float v6 = a6 * 4398046511104.f;
+    const float t = fmaf(v6, 1.f / 4096.f, kMagic);
+    const float r = fmaf(t - kMagic, -4096.f, v6) + kMagic;
+    const int z = (int)((__float_as_uint(t) - kMagicBits) << 14) + (int)((__float_as_uint(r) - kMagicBits) << 2) +
+                  (int)(__float_as_uint(fmaf(a7, 17592186044416.f, kMagic)) - kMagicBits);
+    // (l4 << 16) + (l5 << 9) + z
+    const unsigned int x = (unsigned int)l4 << 16, s = x + ((unsigned int)l5 << 9), lo = s + (unsigned int)z;
     const unsigned int hi = (unsigned int)(l4 >> 16) + (unsigned int)(l5 >> 23) + (unsigned int)(z >> 31) +
                             (s < x ? 1u : 0u) + (lo < s ? 1u : 0u);
     return make_uint2(lo, hi);
@@ -240,7 +280,6 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
     uint32_t* tmem_slot = (uint32_t*)(drain + 1);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (L.flags[0]) return;  // (written by earlier kernels only: uniform over the grid)
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2 * kStages; ++i) mbar_init(smem_u32(&full_bar[i]), 1);
@@ -257,8 +296,12 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
     const uint32_t tmem = *tmem_slot;
     Walk walk(L);
     Segment g;
+    grid_dependency_wait();
+    // a step that is not taken (written by earlier kernels only: uniform over the grid)
+    const bool skip = L.flags[0] != 0;
 
-    if (warp == 0) {
+    if (skip) {
+    } else if (warp == 0) {
         if (lane == 0) {
             int it = 0;
             bool ok = true;
@@ -400,13 +443,16 @@ __device__ __forceinline__ V row_reduce(V v, Op op) {
 }
 
 // TPR threads per row (a warp for short rows, the block of 256 for long ones),
-// four consecutive columns each.  Bound by HBM (8 bytes read and 16 written
-// per element): a row is read three times, the second and third time from L1.
+// NG groups of four consecutive columns per thread, held in registers between
+// the three passes over the row (largest exponent, 2-norm, digits); NG = 0:
+// longer rows, read again from L1 / L2 by each pass.  Bound by HBM for large n (8
+// bytes read and 16 written per element), by load latency for small n.
 // Integer arithmetic and float32 only.
-template <int TPR>
+template <int TPR, int NG>
 __global__ void __launch_bounds__(256)
 f64_split_kernel(const double* __restrict__ X, int n, int n_pad, __nv_bfloat16* __restrict__ planes,
                  int* __restrict__ exps, int* flags, int step) {
+    grid_dependency_wait();
     // (a block of this launch may set it: decide once per block)
     if (__syncthreads_or(*(volatile int*)flags != 0)) return;
     const int i = (int)blockIdx.x * (256 / TPR) + (int)threadIdx.x / TPR;  // < n_pad, a multiple of 128
@@ -428,25 +474,37 @@ f64_split_kernel(const double* __restrict__ X, int n, int n_pad, __nv_bfloat16* 
                 if (j0 + c < n) x[c] = row[j0 + c];
         }
     };
+    double held[NG > 0 ? NG : 1][4];
+    if constexpr (NG > 0) {
+#pragma unroll
+        for (int g = 0; g < NG; ++g) load4(4 * (t + g * TPR), held[g]);
+    }
+    auto for_row = [&](int end, auto&& body) {
+        if constexpr (NG > 0) {
+#pragma unroll
+            for (int g = 0; g < NG; ++g)
+                if (4 * (t + g * TPR) < end) body(4 * (t + g * TPR), held[g]);
+        } else {
+            for (int j0 = 4 * t; j0 < end; j0 += 4 * TPR) {
+                load4(j0, held[0]);
+                body(j0, held[0]);
+            }
+        }
+    };
     unsigned int top = 0;  // the largest high word: sign off, exponent and 20 leading bits
-    unsigned int low = 0;  // whether a low word is set where the high word is zero
-    for (int j0 = 4 * t; j0 < n; j0 += 4 * TPR) {
-        double x[4];
-        load4(j0, x);
+    unsigned int low = 0;  // the low words' bits
+    for_row(n, [&](int, double (&x)[4]) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             top = max(top, (unsigned int)__double2hiint(x[c]) & 0x7fffffffu);
             low |= (unsigned int)__double2loint(x[c]);
         }
-    }
+    });
     top = row_reduce<TPR>(top, [](unsigned int a, unsigned int b) { return max(a, b); });
-    low = row_reduce<TPR>(low, [](unsigned int a, unsigned int b) { return a | b; });
     const int emax = (int)(top >> 20);
     // sum of squares relative to 2^(emax - 1023), from the high words
     float ss = 0.f;
-    for (int j0 = 4 * t; j0 < n; j0 += 4 * TPR) {
-        double x[4];
-        load4(j0, x);
+    for_row(n, [&](int, double (&x)[4]) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const unsigned int h = (unsigned int)__double2hiint(x[c]) & 0x7fffffffu;
@@ -454,20 +512,19 @@ f64_split_kernel(const double* __restrict__ X, int n, int n_pad, __nv_bfloat16* 
             const float m = d > -60 ? __uint_as_float((unsigned int)(127 + d) << 23 | (h & 0xfffffu) << 3) : 0.f;
             ss = fmaf(m, m, ss);
         }
-    }
+    });
     ss = row_reduce<TPR>(ss, [](float a, float b) { return a + b; });
     // the smallest k with 4^k > ss (raised by the truncation and the sum's rounding)
     const int lg = (int)(__float_as_uint(ss * 1.01f) >> 23) - 127;
     const int e = emax == 0 ? 0 : emax - 1023 + ((lg + 2) >> 1);
     // outside the digits' range: not finite, denormal, or a scale beyond 2^+-400
-    const bool bad = emax == 0 ? (top | low) != 0 : (emax == 2047 || e > kExpLimit || e < -kExpLimit);
-    if (t == 0) {
-        exps[i] = e;
-        if (bad) atomicCAS(flags, 0, step + 1);
+    if (emax == 0) {
+        if ((top | low) != 0) atomicCAS(flags, 0, step + 1);
+    } else if (t == 0 && (emax == 2047 || e > kExpLimit || e < -kExpLimit)) {
+        atomicCAS(flags, 0, step + 1);
     }
-    for (int j0 = 4 * t; j0 < n_pad; j0 += 4 * TPR) {
-        double x[4];
-        load4(j0, x);
+    if (t == 0) exps[i] = e;
+    for_row(n_pad, [&](int j0, double (&x)[4]) {
         uint32_t w[kDigits][2];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -515,7 +572,7 @@ f64_split_kernel(const double* __restrict__ X, int n, int n_pad, __nv_bfloat16* 
 #pragma unroll
         for (int p = 0; p < kDigits; ++p)
             *(uint2*)(planes + quad_index(p, i, j0, n_pad)) = make_uint2(w[p][0], w[p][1]);
-    }
+    });
 }
 
 // ---- finish: fixed-point product -> the step's polynomial ----------------------
@@ -526,92 +583,150 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-// Y = cP P + cE E + cI I, C = dY Y + dI I (with mirror) over the 32 x 32 blocks
-// I <= J, and the reductions of step_f64_kernel.  Reads each fixed-point entry
-// once and clears it for the next step.
-__global__ void __launch_bounds__(256)
-f64_finish_kernel(unsigned long long* __restrict__ T, const int* __restrict__ ea, const int* __restrict__ eb,
-                  const double* __restrict__ E, double* __restrict__ C, int n, int blocks, double cP, double cE,
+// v 2^ex, rounded to nearest even (|ex| < 900, |v| < 2^63): integer operations
+// on 32-bit halves, where a conversion and a multiplication would take the
+// float64 pipe.
+__device__ __forceinline__ double fixed_to_double(uint2 v, int ex) {
+    const unsigned int sign = v.y & 0x80000000u;
+    unsigned int lo = v.x, hi = v.y;
+    if (sign) {
+        lo = 0u - lo;
+        hi = ~hi + (lo == 0u ? 1u : 0u);
+    }
+    if ((lo | hi) == 0u) return 0.0;
+    const int z = hi ? __clz(hi) : 32 + __clz(lo);
+    if (z >= 32) {
+        hi = lo;
+        lo = 0u;
+    }
+    hi = __funnelshift_l(lo, hi, z);  // (shifts by z mod 32)
+    lo <<= z & 31;
+    // bit 63 leads: 53 bits kept, ties to even
+    const unsigned int rem = lo & 0x7ffu, mlo = hi << 21 | lo >> 11;
+    const unsigned int inc = (rem > 0x400u || (rem == 0x400u && (mlo & 1u))) ? 1u : 0u;
+    const unsigned int rlo = mlo + inc;
+    const unsigned int rhi = (hi >> 11) + (rlo < inc ? 1u : 0u) + ((unsigned int)(63 - z + ex + 1022) << 20);
+    return __hiloint2double((int)(sign | rhi), (int)rlo);
+}
+
+// One pass of a finish block over 32 rows (lane: i = i0 + tx) x 8 NQ columns from
+// j0 of the 32 x 32 block (I, J); DIAG: I = J.  The diagonal's extra terms are
+// kept out of the other blocks' code: an instruction whose predicate is off
+// still takes its turn on the float64 pipe.
+template <int NQ, bool HAS_E, bool AFFINE, bool DIAG>
+__device__ __forceinline__ void finish_pass(const uint2 (&v)[NQ], const double (&e)[NQ], const int (&ex)[NQ], int i,
+                                            int j0, int n, double* __restrict__ C, double cP, double cE, double cI,
+                                            double dY, double dI, double (*tile)[33], double& s_tr, double& s_idem) {
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    double sd = 0.0;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        const int c = ty + 8 * q, j = j0 + c;
+        double out = 0.0;
+        if (i < n && j < n && (!DIAG || i <= j)) {
+            const double p = fixed_to_double(v[q], ex[q]);
+            double y = cP * p;
+            if (HAS_E) {
+                y = fma(cE, e[q], y);
+                const double d = e[q] - p;
+                sd = fma((DIAG && i == j) ? 0.5 * d : d, d, sd);
+            }
+            if (DIAG && i == j) y += cI;
+            out = y;
+            if (AFFINE) out = dY * y;
+            if (DIAG && i == j) {
+                out += dI;
+                s_tr += y;
+            }
+            C[(size_t)j * n + i] = out;
+        }
+        tile[c][tx] = out;
+    }
+    if (HAS_E) s_idem += sd;  // half of the sum over the whole matrix
+}
+
+// Y = cP P + cE E + cI I, C = dY Y + dI I (with mirror) over pieces of the 32 x
+// 32 blocks I <= J: 32 rows x 8 NQ columns per pass of a block of threads.
+// red[0] += trace(Y), red[1] += ||E - P||_F^2 (HAS_E).  Reads each fixed-point
+// entry once and clears it for the next step.  At most four float64
+// operations per element of the upper triangle: at n = 4096 they take 60 us of
+// that pipe, the 40 bytes per upper element 50 us of HBM; 185 us measured (372
+// with conversions and the diagonal's terms on the float64 pipe).  NQ = 1
+// spreads small matrices over more SMs (n = 256: 36 blocks of 32 x 32).
+template <int NQ, bool HAS_E, bool AFFINE>
+__global__ void __launch_bounds__(256, 5)
+f64_finish_kernel(uint2* __restrict__ T, const int* __restrict__ ea, const int* __restrict__ eb,
+                  const double* __restrict__ E, double* __restrict__ C, int n, int pieces, double cP, double cE,
                   double cI, double dY, double dI, double* red, const int* __restrict__ flags) {
-    __shared__ double tile[32][33];
-    __shared__ double rsum[3][8];
+    constexpr int PB = 4 / NQ;  // pieces per 32 x 32 block
+    __shared__ double tile[8 * NQ][33];
+    __shared__ double rsum[256];
+    grid_dependency_wait();
     if (flags[0]) return;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    double s_tr = 0.0, s_idem = 0.0, s_fro = 0.0;
-    const bool affine = dY != 1.0 || dI != 0.0;
-    for (int b = blockIdx.x; b < blocks; b += gridDim.x) {
+    double s_tr = 0.0, s_idem = 0.0;
+    bool any_diag = false;
+    for (int u = blockIdx.x; u < pieces; u += gridDim.x) {
+        const int b = u / PB, c0 = (u % PB) * 8 * NQ;
         int J = (int)((sqrtf(8.f * (float)b + 1.f) - 1.f) * 0.5f);
         while ((J + 1) * (J + 2) / 2 <= b) ++J;
         while (J * (J + 1) / 2 > b) --J;
         const int I = b - J * (J + 1) / 2;
-        unsigned long long* t = T + (size_t)((J >> 2) * ((J >> 2) + 1) / 2 + (I >> 2)) * (TILE * TILE) +
-                                (size_t)((J & 3) * 32) * TILE + (I & 3) * 32 + tx;
-        const int i = I * 32 + tx;
-        const int ei = ea[i];
-        unsigned long long v[4];
-        double e[4];
+        uint2* t = T + (size_t)((J >> 2) * ((J >> 2) + 1) / 2 + (I >> 2)) * (TILE * TILE) +
+                   (size_t)((J & 3) * 32 + c0) * TILE + (I & 3) * 32 + tx;
+        const int i = I * 32 + tx, j0 = J * 32 + c0;
+        const int ei = ea[i] - 60;
+        uint2 v[NQ];
+        double e[NQ];
+        int ex[NQ];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = ty + 8 * q, j = J * 32 + c;
+        for (int q = 0; q < NQ; ++q) {
+            const int c = ty + 8 * q, j = j0 + c;
             v[q] = t[c * TILE];
-            t[c * TILE] = 0ull;
-            e[q] = (E && i < n && j < n) ? E[(size_t)j * n + i] : 0.0;
+            e[q] = (HAS_E && i < n && j < n) ? E[(size_t)j * n + i] : 0.0;
+            ex[q] = ei + eb[j];
         }
-        double sd = 0.0, sf = 0.0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = ty + 8 * q, j = J * 32 + c;
-            double out = 0.0;
-            if (i < n && j < n && i <= j) {
-                const double p = (double)(long long)v[q] * __hiloint2double((ei + eb[j] - 60 + 1023) << 20, 0);
-                double y = cP * p + cE * e[q];
-                if (i == j) y += cI;
-                out = y;
-                if (affine) out = dY * y;
-                if (i == j) {
-                    out += dI;
-                    s_tr += y;
-                }
-                C[(size_t)j * n + i] = out;
-                if (red) {
-                    const double d = e[q] - p;
-                    double d2 = d, y2 = y;
-                    if (I == J && i != j) {  // (off-diagonal blocks are doubled below)
-                        d2 += d;
-                        y2 += y;
-                    }
-                    sd = fma(d2, d, sd);
-                    sf = fma(y2, y, sf);
-                }
-            }
-            tile[c][tx] = out;
+        for (int q = 0; q < NQ; ++q) t[(ty + 8 * q) * TILE] = make_uint2(0u, 0u);
+        if (I == J) {
+            any_diag = true;
+            finish_pass<NQ, HAS_E, AFFINE, true>(v, e, ex, i, j0, n, C, cP, cE, cI, dY, dI, tile, s_tr, s_idem);
+        } else {
+            finish_pass<NQ, HAS_E, AFFINE, false>(v, e, ex, i, j0, n, C, cP, cE, cI, dY, dI, tile, s_tr, s_idem);
         }
-        const double wb = I == J ? 1.0 : 2.0;
-        s_idem += wb * sd;
-        s_fro += wb * sf;
         __syncthreads();
+        // the row segments (i, j0 .. j0 + 8 NQ): 8 NQ threads a row
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int r = ty + 8 * q, i2 = I * 32 + r, j2 = J * 32 + tx;
-            if (i2 < n && j2 < n && i2 < j2) C[(size_t)i2 * n + j2] = tile[tx][r];
+        for (int q = 0; q < NQ; ++q) {
+            const int w = threadIdx.x + 256 * q, r = w / (8 * NQ), c = w % (8 * NQ);
+            const int i2 = I * 32 + r, j2 = j0 + c;
+            if (j2 < n && i2 < j2) C[(size_t)i2 * n + j2] = tile[c][r];
         }
         __syncthreads();
     }
-    if (red) {
-        s_tr = warp_sum_d(s_tr);
-        s_idem = warp_sum_d(s_idem);
-        s_fro = warp_sum_d(s_fro);
-        if (tx == 0) {
-            rsum[0][ty] = s_tr;
-            rsum[1][ty] = s_idem;
-            rsum[2][ty] = s_fro;
+    if (!red) return;
+    // one warp adds up the block (a shuffle tree in every warp would put eight
+    // times as many additions on the float64 pipe); the trace only where the
+    // block met the diagonal
+    auto block_total = [&](double x) -> double {
+        rsum[threadIdx.x] = x;
+        __syncthreads();
+        double w = 0.0;
+        if (ty == 0) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) w += rsum[tx + 32 * q];
+            w = warp_sum_d(w);
         }
         __syncthreads();
-        if (threadIdx.x < 3) {
-            double v = 0.0;
-            for (int q = 0; q < 8; ++q) v += rsum[threadIdx.x][q];
-            atomicAdd(&red[threadIdx.x], v);
-        }
+        return w;
+    };
+    if (HAS_E) {
+        const double w = block_total(s_idem);
+        if (threadIdx.x == 0) atomicAdd(&red[1], 2.0 * w);
+    }
+    if (any_diag) {
+        const double w = block_total(s_tr);
+        if (threadIdx.x == 0) atomicAdd(&red[0], w);
     }
 }
 
@@ -666,11 +781,14 @@ bool f64d_begin(F64Digits& f, int64_t n, int operands, cudaStream_t s, int* err)
 }
 
 static int split_into(F64Digits& f, int b, const double* X, int64_t n, cudaStream_t s) {
-    if (n <= 1024)
-        f64_split_kernel<32><<<f.n_pad / 8, 256, 0, s>>>(X, (int)n, f.n_pad, f.planes[b], f.exps[b], f.flags, f.step);
-    else
-        f64_split_kernel<256><<<f.n_pad, 256, 0, s>>>(X, (int)n, f.n_pad, f.planes[b], f.exps[b], f.flags, f.step);
-    PURIFY_CUDA_TRY(cudaGetLastError());
+    auto go = [&](auto kernel, int rows_per_block) {
+        return launch_chained(kernel, (unsigned)(f.n_pad / rows_per_block), 256u, 0, s, X, (int)n, f.n_pad, f.planes[b],
+                              f.exps[b], f.flags, f.step);
+    };
+    PURIFY_CUDA_TRY(n <= 512    ? go(f64_split_kernel<32, 4>, 8)
+                    : n <= 1024 ? go(f64_split_kernel<256, 1>, 1)
+                    : n <= 4096 ? go(f64_split_kernel<256, 4>, 1)
+                                : go(f64_split_kernel<256, 0>, 1));
     count_launches(1);
     f.held[b] = X;
     return PURIFY_OK;
@@ -706,11 +824,22 @@ int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, d
         const long long cost = (long long)L.tiles * L.tiles_per_row * 4 * kCost32;
         grid = (int)std::max<long long>(1, std::min<long long>(grid, cost / kMinCost));
     }
-    f64_digit_product_kernel<<<grid, kThreads, kSmemBytes, s>>>(L);
+    PURIFY_CUDA_TRY(launch_chained(f64_digit_product_kernel, (unsigned)grid, (unsigned)kThreads, kSmemBytes, s, L));
     const int64_t nb = (n + 31) / 32, blocks = nb * (nb + 1) / 2;
-    f64_finish_kernel<<<(unsigned)std::min<int64_t>(blocks, (int64_t)f.ctas * 8), 256, 0, s>>>(
-        f.T, f.exps[a], f.exps[b], E, C, (int)n, (int)blocks, cP, cE, cI, dY, dI, red, f.flags);
-    PURIFY_CUDA_TRY(cudaGetLastError());
+    auto finish = [&](auto kernel, int64_t pieces) {
+        return launch_chained(kernel, (unsigned)std::min<int64_t>(pieces, (int64_t)f.ctas * 5), 256u, 0, s, (uint2*)f.T,
+                              f.exps[a], f.exps[b], E, C, (int)n, (int)pieces, cP, cE, cI, dY, dI, red, f.flags);
+    };
+    auto finish_nq = [&](auto e, auto affine) {
+        constexpr bool HE = decltype(e)::value, AF = decltype(affine)::value;
+        return blocks < 4 * f.ctas ? finish(f64_finish_kernel<1, HE, AF>, 4 * blocks)
+                                   : finish(f64_finish_kernel<4, HE, AF>, blocks);
+    };
+    const bool affine = dY != 1.0 || dI != 0.0;
+    PURIFY_CUDA_TRY(E ? (affine ? finish_nq(std::true_type(), std::true_type())
+                                : finish_nq(std::true_type(), std::false_type()))
+                      : (affine ? finish_nq(std::false_type(), std::true_type())
+                                : finish_nq(std::false_type(), std::false_type())));
     count_launches(2);
     for (int q = 0; q < 2; ++q)
         if (f.held[q] == C) f.held[q] = nullptr;

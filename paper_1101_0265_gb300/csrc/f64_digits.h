@@ -29,7 +29,8 @@ bool f64d_wanted(int64_t n);
 // receives other failures.
 bool f64d_begin(F64Digits& f, int64_t n, int operands, cudaStream_t s, int* err);
 
-// launch_step_f64 by exact digit products; A, B and E are exactly symmetric.
+// launch_step_f64 by exact digit products (red[2] is not reduced); A, B and E are
+// exactly symmetric.
 int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, double* C, int64_t n, double cP,
               double cE, double cI, double dY, double dI, double* red, cudaStream_t s);
 
