@@ -1,6 +1,7 @@
 // Host side of the digit-plane products: the float64 -> digit-plane split
 // kernel, tensor maps, kernel choice and launch.  The product kernel itself
 // is in digits_kernel.cuh (instantiated in digits_k*.cu).
+#include "digits_fixed.h"
 #include "digits_kernel.cuh"
 
 #include <algorithm>
@@ -419,7 +420,7 @@ int prepare_digit_kernels() {
         PURIFY_TRY(prepare_kernel(queue_kernel(s, true)));
         PURIFY_TRY(prepare_kernel(s <= 3 ? kernel_pool_lo(s) : kernel_pool_hi(s)));
     }
-    return PURIFY_OK;
+    return prepare_digit_fixed();
 }
 
 int fill_digit_params(const DigitStep& st, DigitGemmParams* p, CUtensorMap* ma, CUtensorMap* mb) {
@@ -504,7 +505,29 @@ void digit_split_plan(int tiles, int ctas, int k_chunks, int* split_begin, int* 
     *ways = w;
 }
 
+void digit_step_split(const DigitStep& st, int tiles, int* split_begin, int* ways) {
+    *split_begin = tiles;
+    *ways = 1;
+    if (!st.partial || !st.split_cnt || st.kc_cnt || st.split_ways == 1) return;
+    const int nk = st.n_pad / digit_step_kc(st);
+    digit_split_plan(tiles, st.max_ctas, nk, split_begin, ways);
+    if (st.split_ways > 1 && *ways > 1) {
+        // a chosen number of ranges: at most 4, each of at least 4 k-chunks,
+        // and at most max_ctas parts in all (the partial buffer holds
+        // digit_partial_floats(max_ctas))
+        const int tail = tiles - *split_begin;
+        int w = st.split_ways < 4 ? st.split_ways : 4;
+        while (w > 1 && (nk / w < 4 || tail * w > st.max_ctas)) --w;
+        *ways = w;
+    }
+    if (*ways < 2) {
+        *split_begin = tiles;
+        *ways = 1;
+    }
+}
+
 int launch_digit_step(const DigitStep& st, cudaStream_t stream) {
+    if (digits_fixed_wanted(st)) return launch_digit_fixed(st, stream);
     DigitLaunch L;
     std::memset(&L, 0, sizeof(L));
     PURIFY_TRY(fill_digit_params(st, &L.prms[0], &L.maps[0], &L.maps[1]));
@@ -517,25 +540,7 @@ int launch_digit_step(const DigitStep& st, cudaStream_t stream) {
     L.err = st.err;
     L.wait_cycles = st.wait_cycles;
     if (!st.scratch || !st.err) return PURIFY_ERR_INVALID_ARG;
-    L.split_begin = tiles;
-    L.split_ways = 1;
-    if (st.partial && st.split_cnt && !st.kc_cnt && st.split_ways != 1) {
-        digit_split_plan(tiles, st.max_ctas, st.n_pad / kc, &L.split_begin, &L.split_ways);
-        if (st.split_ways > 1 && L.split_ways > 1) {
-            // a chosen number of ranges: at most 4, each of at least 4
-            // k-chunks, and at most max_ctas parts in all (the partial buffer
-            // holds digit_partial_floats(max_ctas))
-            const int tail = tiles - L.split_begin;
-            int w = st.split_ways < 4 ? st.split_ways : 4;
-            while (w > 1 && ((st.n_pad / kc) / w < 4 || tail * w > st.max_ctas)) --w;
-            L.split_ways = w;
-            if (w < 2) L.split_begin = tiles;
-        }
-    }
-    if (L.split_ways < 2) {
-        L.split_begin = tiles;
-        L.split_ways = 1;
-    }
+    digit_step_split(st, tiles, &L.split_begin, &L.split_ways);
     L.num_items = L.split_begin + (tiles - L.split_begin) * L.split_ways;
     if (L.split_ways > 1 && (tiles - L.split_begin) * L.split_ways > st.max_ctas) return PURIFY_ERR_INVALID_ARG;
     if (L.split_ways > 1) {

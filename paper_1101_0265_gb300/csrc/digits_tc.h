@@ -38,6 +38,17 @@ __host__ __device__ inline size_t plane_index(int p, int i, int j, int n_pad) {
 // Bytes of a buffer of s digit planes at size n_pad.
 inline size_t plane_buffer_bytes(int s, int n_pad) { return (size_t)plane_pairs(s) * 2 * n_pad * n_pad * 2; }
 
+// Device buffers of a small product's sums (digits_fixed.cu): levels 0 to 2 as
+// integers, of whole tiles and of tiles summed in parts (zero before and after
+// a step), the shared accumulator of levels >= 3 by work item, and a flag that
+// poisons the run.
+struct FixedSums {
+    unsigned long long* levels = nullptr;
+    unsigned long long* parts = nullptr;
+    float* shared = nullptr;
+    int* poison = nullptr;
+};
+
 // One fused step: P = A B (A, B symmetric, held as s_in digit planes each,
 // scale exponents eA, eB), Y = cP P + cE E + cI I with E = A when use_E,
 // out = dY Y + dI I written as s_out digit planes with exponent e_out and
@@ -86,6 +97,9 @@ struct DigitStep {
     const int* b_idx = nullptr;
     const int* out_idx = nullptr;
     int a_slots = 0, b_slots = 0;
+    // buffers of the two-launch path of small products (digits_fixed.cu); null:
+    // the persistent kernel
+    const FixedSums* fixed = nullptr;
     // device-side control (null: the fields above decide)
     const DevStep* ctl = nullptr;
 };
@@ -105,6 +119,9 @@ void digit_split_plan(int tiles, int ctas, int k_chunks, int* split_begin, int* 
 inline size_t digit_scratch_bytes(int ctas) { return (size_t)ctas * 128 * 128 * sizeof(float2); }
 
 int launch_digit_step(const DigitStep& st, cudaStream_t stream);
+// The split of a single dense step's tiles: [0, split_begin) whole, the others
+// in `ways` k-ranges each.
+void digit_step_split(const DigitStep& st, int tiles, int* split_begin, int* ways);
 
 // Opt every product-kernel instantiation into the full shared memory (once
 // per process; call before capturing launches into a graph).

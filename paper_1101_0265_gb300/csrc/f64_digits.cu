@@ -55,6 +55,7 @@
 #include <type_traits>
 
 #include "digits_kernel.cuh"
+#include "tile_sums.cuh"
 
 namespace purify {
 
@@ -91,30 +92,6 @@ struct F64Product {
     int* flags;
     int tiles_per_row, tiles, whole;  // whole: full waves of tiles
 };
-
-// Launched with programmatic stream serialization: the kernel's prologue runs
-// beside its predecessor's tail; memory is touched only after the
-// predecessor has completed, and the successor may then start its own prologue.
-__device__ __forceinline__ void grid_dependency_wait() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-template <typename... KArgs, typename... Args>
-cudaError_t launch_chained(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
-                           Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at = {};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
-}
 
 // The segments of one CTA, the same sequence in every role: a tile, a pass and
 // a run of stages.
@@ -212,27 +189,6 @@ __device__ __forceinline__ void issue_low(uint32_t tmem, uint64_t da, uint64_t d
         mma_bf16(tmem + (uint32_t)(3 * TILE), da + (uint64_t)quad_off(p), db + (uint64_t)quad_off(8 - p), IDESC, 1u);
 }
 
-// 8 columns of the four accumulators, 32 lanes each; tmem_wait32 orders the
-// registers' use after the loads.
-__device__ __forceinline__ void tmem_issue32(uint32_t taddr, uint32_t (&r)[32]) {
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                     : "=r"(r[8 * a]), "=r"(r[8 * a + 1]), "=r"(r[8 * a + 2]), "=r"(r[8 * a + 3]),
-                       "=r"(r[8 * a + 4]), "=r"(r[8 * a + 5]), "=r"(r[8 * a + 6]), "=r"(r[8 * a + 7])
-                     : "r"(taddr + (uint32_t)(a * TILE)));
-}
-
-__device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
-                   "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
-                   "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28])
-                 :: "memory");
-    asm volatile("" : "+r"(r[29]), "+r"(r[30]), "+r"(r[31])::"memory");
-}
-
 // The four accumulators of one element as a 64-bit integer in units of
 // 2^-60, modulo 2^64: 32-bit halves (64-bit integer operations run on the
 // float64 pipe).  Conversions of floats to integers run at 16 per clock and SM,
@@ -240,9 +196,6 @@ __device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32]) {
 // 2^22 (0 and 1: |L_1| <= 2 x 2^8 x 64 x 32; 7 in units of 32) are read off the
 // bits of a sum with 1.5 2^23 instead, and one of the larger low levels in two
 // such pieces.
-constexpr float kMagic = 12582912.f;  // 1.5 2^23: bits 0x4B400000
-constexpr unsigned int kMagicBits = 0x4B400000u;
-
 __device__ __forceinline__ uint2 levels_high(float a0, float a1, float a2, float a3) {
     const unsigned int l0 = __float_as_uint(a0 + kMagic), l1 = __float_as_uint(fmaf(a1, 128.f, kMagic));
     const int l2 = __float2int_rn(a2 * 16384.f), l3 = __float2int_rn(a3 * 2097152.f);
@@ -399,6 +352,8 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
                     if (lane == 0)
                         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(tmem_empty)) : "memory");
                 }
+                // blocks below the diagonal are the mirror of others
+                if (g.ti == g.tj && quarter > ((col0 + 8 * q) >> 5)) continue;
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     const float a0 = __uint_as_float(v[c]), a1 = __uint_as_float(v[8 + c]),
@@ -764,7 +719,8 @@ bool f64d_begin(F64Digits& f, int64_t n, int operands, cudaStream_t s, int* err)
         for (int b = 0; b < operands; ++b) PURIFY_TRY(ensure_planes(f, b));
         PURIFY_CUDA_TRY(cudaFuncSetAttribute((const void*)f64_digit_product_kernel,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-        PURIFY_CUDA_TRY(cudaMemsetAsync(f.T, 0, t_bytes(n_pad), s));
+        if (!f.clean) PURIFY_CUDA_TRY(cudaMemsetAsync(f.T, 0, t_bytes(f.cap_pad), s));
+        f.clean = false;
         PURIFY_CUDA_TRY(cudaMemsetAsync(f.flags, 0, 2 * sizeof(int), s));
         return PURIFY_OK;
     };
@@ -854,6 +810,7 @@ int f64d_check(F64Digits& f, cudaStream_t s, int* redo_from) {
     PURIFY_CUDA_TRY(cudaStreamSynchronize(s));
     if (v[1]) return PURIFY_ERR_DEVICE_TIMEOUT;
     *redo_from = v[0] - 1;
+    f.clean = v[0] == 0;
     return PURIFY_OK;
 }
 

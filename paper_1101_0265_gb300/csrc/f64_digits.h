@@ -15,6 +15,7 @@ struct F64Digits {
     __nv_bfloat16* planes[2] = {nullptr, nullptr};
     int* exps[2] = {nullptr, nullptr};  // row exponents of planes[b]
     unsigned long long* T = nullptr;    // fixed-point product, upper 128 x 128 tiles; zero between steps
+    bool clean = false;                 // T is zero (the last run ended well)
     int* flags = nullptr;  // [0] the step (from 1) whose operand left the digits' range; [1] a wait that ran out
     const double* held[2] = {nullptr, nullptr};  // the run's matrix whose digits planes[b] hold
     int step = 0;                                // steps queued since f64d_begin

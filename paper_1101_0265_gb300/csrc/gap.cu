@@ -335,7 +335,7 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
     if (mixed) {
         PURIFY_TRY(ensure_mixed(h, n_pad));
         PURIFY_TRY(launch_split(h->F, n, (int)n, n_pad, c1, c0, 0, kMaxDigitPlanes, rb, h->mixed->Xd[0], nullptr, s));
-        PURIFY_CUDA_TRY(cudaMemsetAsync(h->mixed->err, 0, sizeof(int), s));
+        PURIFY_TRY(begin_products(h, n_pad));
     } else {
         PURIFY_TRY(launch_affine_f64(h->F, n, Xf[1], n, c1, c0, s));
     }
@@ -392,11 +392,7 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
             st.err = ms->err;
             st.scratch = ms->scratch;
             st.max_ctas = ms->ctas;
-            if (h->opt.split_k) {
-                st.partial = ms->partial;
-                st.split_cnt = ms->split_cnt;
-            }
-            st.wait_cycles = 1000ll * h->opt.wait_kcycles;
+            attach_products(h, &st);
             r = launch_digit_step(st, s);
         } else {
             const double* Xi = Xf[(i + 1) & 1];
@@ -465,6 +461,7 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
     }
     h->st.device_flag = err;
     if (err) return device_flag_status(err);
+    if (mixed) end_products(h);
     if (rc == PURIFY_OK) {
         h->b.homo = homo;
         h->b.lumo = lumo;

@@ -9,6 +9,7 @@
 // mapped gap g_i: the smallest s in [3, 6] whose digits carry
 // max(30, 26 + log2(1 / g_i)) bits (8 + 7 (s - 1) bits up to n = 4096), so
 // early steps (small g) carry 43 bits and late ones 36.
+#include "digits_fixed.h"
 #include "mixed.h"
 
 #include <algorithm>
@@ -42,6 +43,7 @@ void mixed_free(MixedState* ms) {
     cudaFree(ms->tsel);
     cudaFree(ms->tsched);
     cudaFree(ms->qdev);
+    free_fixed_sums(&ms->fixed);
     for (int k = 0; k < 2; ++k) {
         cudaFree(ms->pool[k]);
         cudaFree(ms->pidx[k]);
@@ -59,7 +61,7 @@ int ensure_mixed(purify_ctx* h, int n_pad, bool planes) {
     if (!h->mixed) {
         h->mixed = new (std::nothrow) MixedState();
         if (!h->mixed) return PURIFY_ERR_OOM;
-        PURIFY_CUDA_TRY(cudaMalloc(&h->mixed->err, sizeof(int)));
+        PURIFY_CUDA_TRY(cudaMalloc(&h->mixed->err, 2 * sizeof(int)));
         int sms = 0;
         PURIFY_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
         h->mixed->ctas = sms;
@@ -80,6 +82,38 @@ int ensure_mixed(purify_ctx* h, int n_pad, bool planes) {
     PURIFY_CUDA_TRY(cudaMalloc(&ms->Sd, bytes));
     ms->n_pad_cap = n_pad;
     return PURIFY_OK;
+}
+
+int begin_products(purify_ctx* h, int n_pad) {
+    MixedState* ms = h->mixed;
+    // [0] the product kernels' error bits, [1] a fixed-point sum out of range
+    PURIFY_CUDA_TRY(cudaMemsetAsync(ms->err, 0, 2 * sizeof(int), h->stream));
+    if (!digits_fixed_size(n_pad, ms->ctas)) return PURIFY_OK;
+    if (!ms->fixed.shared) {
+        ms->fixed_clean = false;
+        if (alloc_fixed_sums(ms->ctas, &ms->fixed) != PURIFY_OK) {
+            free_fixed_sums(&ms->fixed);  // no room: the persistent kernel needs none
+            cudaGetLastError();
+            return PURIFY_OK;
+        }
+        ms->fixed.poison = ms->err + 1;
+    }
+    if (!ms->fixed_clean)
+        PURIFY_CUDA_TRY(cudaMemsetAsync(ms->fixed.parts, 0, digits_fixed_part_bytes(ms->ctas), h->stream));
+    ms->fixed_clean = false;
+    return PURIFY_OK;
+}
+
+void end_products(purify_ctx* h) { h->mixed->fixed_clean = h->mixed->fixed.shared != nullptr; }
+
+void attach_products(purify_ctx* h, DigitStep* st) {
+    MixedState* ms = h->mixed;
+    if (h->opt.split_k) {
+        st->partial = ms->partial;
+        st->split_cnt = ms->split_cnt;
+    }
+    if (ms->fixed.shared) st->fixed = &ms->fixed;
+    st->wait_cycles = 1000ll * h->opt.wait_kcycles;
 }
 
 // Digits for a step whose mapped gap (distance between the images of the
@@ -204,11 +238,7 @@ void tuned_shape_if_known(int device, DigitStep* st) {
 
 static int product(purify_ctx* h, const DigitStep& st0, double flops) {
     DigitStep st = st0;
-    if (h->opt.split_k) {
-        st.partial = h->mixed->partial;
-        st.split_cnt = h->mixed->split_cnt;
-    }
-    st.wait_cycles = 1000ll * h->opt.wait_kcycles;
+    attach_products(h, &st);
     if (h->opt.autotune && h->opt.wait_kcycles == 0 && !st.kc_cnt && !st.bnorm2 && st.kc == 0) {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         const auto key = std::make_tuple(h->device, st.s_in, st.n_pad);
@@ -255,7 +285,7 @@ int run_mixed_trace(purify_ctx* h, int scheme, double tol, int max_iter, Schedul
     // slots 0 .. max_iter - 1: the steps; slot max_iter: trace(F)
     PURIFY_TRY(ensure_red(h, 4 * (int64_t)(max_iter + 1)));
     PURIFY_CUDA_TRY(cudaMemsetAsync(h->red, 0, sizeof(double) * 4 * (max_iter + 1), h->stream));
-    PURIFY_CUDA_TRY(cudaMemsetAsync(ms->err, 0, sizeof(int), h->stream));
+    PURIFY_TRY(begin_products(h, n_pad));
     PURIFY_CUDA_TRY(cudaEventRecord(h->e0, h->stream));
     double* trF = h->red + 4 * (int64_t)max_iter;
     PURIFY_TRY(launch_trace_f64(h->F, n, trF, h->stream));
@@ -331,6 +361,7 @@ int run_mixed_trace(purify_ctx* h, int scheme, double tol, int max_iter, Schedul
     PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
     h->st.device_flag = err;
     if (err) return device_flag_status(err);
+    end_products(h);
     if (it == 0) {
         h->st.trace = tr_prev;
         h->st.idem_err_fro = NAN;
@@ -433,7 +464,7 @@ int run_mixed_poly(purify_ctx* h, int scheme, double mu, const Schedule& S, int*
     const int slots = 2 * m + 2;
     PURIFY_TRY(ensure_red(h, 4 * (int64_t)slots));
     PURIFY_CUDA_TRY(cudaMemsetAsync(h->red, 0, sizeof(double) * 4 * slots, h->stream));
-    PURIFY_CUDA_TRY(cudaMemsetAsync(ms->err, 0, sizeof(int), h->stream));
+    PURIFY_TRY(begin_products(h, n_pad));
     PURIFY_CUDA_TRY(cudaEventRecord(h->e0, h->stream));
     const double gamma = std::max((mu - h->b.lmin) / (1.0 - c), (h->b.lmax - mu) / c);
     double* D = h->X[0];
@@ -498,6 +529,7 @@ int run_mixed_poly(purify_ctx* h, int scheme, double mu, const Schedule& S, int*
     PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
     h->st.device_flag = err;
     if (err) return device_flag_status(err);
+    end_products(h);
     h->st.trace = m > 0 ? red[4 * (size_t)(2 * (m - 1) + 1)] : NAN;
     h->st.idem_err_fro = NAN;
     return PURIFY_OK;
@@ -809,7 +841,7 @@ int run_mixed(purify_ctx* h, int scheme, double mu, const Schedule& S, int* cur,
     const int slots = 2 * (m + R) + 2;
     PURIFY_TRY(ensure_red(h, 4 * (int64_t)slots));
     PURIFY_CUDA_TRY(cudaMemsetAsync(h->red, 0, sizeof(double) * 4 * slots, h->stream));
-    PURIFY_CUDA_TRY(cudaMemsetAsync(ms->err, 0, sizeof(int), h->stream));
+    PURIFY_TRY(begin_products(h, n_pad));
     PURIFY_CUDA_TRY(cudaEventRecord(h->e0, h->stream));
 
     const double lmin = h->b.lmin, lmax = h->b.lmax;
@@ -952,6 +984,7 @@ int run_mixed(purify_ctx* h, int scheme, double mu, const Schedule& S, int* cur,
     PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
     h->st.device_flag = err;
     if (err) return device_flag_status(err);
+    end_products(h);
     h->st.refine_multiplications = 2 * R;
     // statistics: trace of the result; idempotency of the last squared iterate
     const int last = m + R - 1;

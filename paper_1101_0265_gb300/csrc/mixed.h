@@ -42,6 +42,10 @@ struct MixedState {
     int pd_cap = 0;
     float* partial = nullptr;   // split last-wave tiles: per-part accumulators
     int* split_cnt = nullptr;   // and per-region arrival counters
+    // small products' sums (digits_fixed.cu); fixed.parts is zero while
+    // fixed_clean
+    FixedSums fixed;
+    bool fixed_clean = false;
     // block-sparse runs: per-tile k-chunk counts, then (8-byte aligned) the
     // per-tile k-chunk bitmasks, in one array of 8-byte words
     unsigned long long* kc_buf = nullptr;
@@ -64,6 +68,7 @@ struct MixedState {
     const double* tg_red = nullptr;
     const double* tg_D = nullptr;
     const void* tg_X0 = nullptr;
+    const void* tg_fixed = nullptr;
     // a whole run as queue launches: staging (host and device copies)
     std::vector<uint8_t> qhost;
     void* qdev = nullptr;
@@ -97,6 +102,14 @@ struct MixedState {
 // Allocate (or grow) the handle's mixed-path buffers for a padded size
 // (planes = false: the state without the dense digit planes).
 int ensure_mixed(purify_ctx* h, int n_pad, bool planes = true);
+// Start a run of single products at size n_pad: clears the device flags and
+// readies the buffers of attach_products.  end_products: the run's flags were
+// read and are clear.
+int begin_products(purify_ctx* h, int n_pad);
+void end_products(purify_ctx* h);
+// The handle's product buffers and options into a step (split_k: the last
+// wave's split, or fixed-point sums where the size wants them).
+void attach_products(purify_ctx* h, DigitStep* st);
 // Default per-step digit rule: a step's operands carry at least kBitsFloor
 // bits and kBitsGap bits beyond log2(1 / mapped gap).
 constexpr double kBitsFloor = 30.0;

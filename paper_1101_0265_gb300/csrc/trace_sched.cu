@@ -178,10 +178,11 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
     PURIFY_TRY(ensure_red(h, 4 * (int64_t)(kBlock + 1)));
     double* red = h->red;
     double* trF = h->red + 4 * kBlock;
+    PURIFY_TRY(begin_products(h, n_pad));
     // captured steps: one block of kBlock steps and a final consume
     const bool key_ok = ms->tgraph && ms->tg_n == n && ms->tg_smin == smin && ms->tg_smax == smax &&
                         ms->tg_state == ms->tsched && ms->tg_red == red && ms->tg_D == h->X[0] &&
-                        ms->tg_X0 == ms->Xd[0] && ms->tg_wait == o.wait_kcycles && ms->tg_split == o.split_k;
+                        ms->tg_X0 == ms->Xd[0] && ms->tg_fixed == ms->fixed.levels && ms->tg_wait == o.wait_kcycles && ms->tg_split == o.split_k;
     if (!key_ok) {
         if (ms->tgraph) cudaGraphExecDestroy(ms->tgraph);
         ms->tgraph = nullptr;
@@ -209,11 +210,7 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
                 st.e_out = 0;
                 st.out64 = h->X[0];
                 st.ctl = &dev->step;
-                st.wait_cycles = 1000ll * o.wait_kcycles;
-                if (o.split_k) {
-                    st.partial = ms->partial;
-                    st.split_cnt = ms->split_cnt;
-                }
+                attach_products(h, &st);
                 tuned_shape_if_known(h->device, &st);
                 rc = launch_digit_step(st, h->stream);
             }
@@ -235,10 +232,10 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
         ms->tg_red = red;
         ms->tg_D = h->X[0];
         ms->tg_X0 = ms->Xd[0];
+        ms->tg_fixed = ms->fixed.levels;
         ms->tg_wait = o.wait_kcycles;
         ms->tg_split = o.split_k;
     }
-    PURIFY_CUDA_TRY(cudaMemsetAsync(ms->err, 0, sizeof(int), h->stream));
     PURIFY_CUDA_TRY(cudaEventRecord(h->e0, h->stream));
     PURIFY_CUDA_TRY(cudaMemcpyAsync(dev, &init, sizeof(init), cudaMemcpyHostToDevice, h->stream));
     PURIFY_CUDA_TRY(cudaMemsetAsync(trF, 0, sizeof(double), h->stream));
@@ -264,6 +261,7 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
     PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
     h->st.device_flag = err;
     if (err) return device_flag_status(err);
+    end_products(h);
     S.alpha.clear();
     S.branch.clear();
     S.beta.clear();
