@@ -120,16 +120,17 @@ struct CsrRows {
     }
 };
 
-// One 32 x 128 strip of the split (see split_kernel); tr accumulates the
-// diagonal's trace (float), the strip's block norms go to bnorm2 when set.
+// Rows [R0, R0 + NR) of one 32 x 128 strip of the split (see split_kernel); tr
+// accumulates the diagonal's trace (float), a whole strip's block norms go to
+// bnorm2 when set.
 // POOLED: the planes go to the pool slots that pidx (nb x nb) gives the
 // blocks (slot 0: not written); a null pidx writes nothing (norms only).
 // `rows` reads F's entries (DenseRows or CsrRows).
-template <bool POOLED, class Rows>
+template <bool POOLED, int NR, class Rows>
 __device__ __forceinline__ void split_strip(const Rows& rows, int n, int n_pad, df a, df b, float digit_scale,
                                             float rscale, float rinv, int s, __nv_bfloat16* __restrict__ out,
                                             float* __restrict__ bnorm2, int strip, int lane, float& tr,
-                                            const int* __restrict__ pidx = nullptr) {
+                                            const int* __restrict__ pidx = nullptr, int r0 = 0) {
     const int nb = n_pad / 32, ns = n_pad / 128;  // nb^2 < 2^27: 32-bit block indices
     const int64_t total = (int64_t)n_pad * n_pad;
     const int I = strip / ns, Jq = strip - I * ns;
@@ -137,9 +138,9 @@ __device__ __forceinline__ void split_strip(const Rows& rows, int n, int n_pad, 
     // the pool slot of this lane's block (I, j0 / 32); 0: not written
     const int slot = (POOLED && pidx) ? pidx[(size_t)I * nb + (j0 >> 5)] : 0;
     float bsum = 0.f;
-#pragma unroll 2
-    for (int r = 0; r < 32; ++r) {  // two rows' loads in flight per warp
-        const int i = I * 32 + r;
+#pragma unroll(NR < 32 ? NR : 2)
+    for (int rr = 0; rr < NR; ++rr) {  // two rows' loads in flight per warp (all of a short piece's)
+        const int r = r0 + rr, i = I * 32 + r;
         double x[4];
         rows(i, j0, lane, x);
         df z[4];
@@ -189,19 +190,27 @@ __device__ __forceinline__ void split_strip(const Rows& rows, int n, int n_pad, 
     }
 }
 
+// Without block norms a warp takes kSplitRows rows of a strip: a whole strip per
+// warp reads 32 rows one after the other, which took 49 us at any small n (n =
+// 200: 16 warps at work) and left loads' latency uncovered at large n.
+constexpr int kSplitRows = 4;
+constexpr int kSplitPieces = 32 / kSplitRows;
+
+template <int NR>
 __global__ void __launch_bounds__(256) split_kernel(const double* __restrict__ F, int64_t ldf, int n, int n_pad,
                                                     df a, df b, float digit_scale, float rscale, int s,
                                                     __nv_bfloat16* __restrict__ out, double* red,
                                                     float* __restrict__ bnorm2) {
+    constexpr int PIECES = 32 / NR;
     const int nb = n_pad / 32, ns = n_pad / 128;
     const int lane = threadIdx.x & 31;
     const int warps = gridDim.x * (blockDim.x >> 5);
     const bool vec = (ldf & 1) == 0 && ((uintptr_t)F & 15) == 0;
     const float rinv = 1.f / rscale;
     float tr = 0.f;
-    for (int strip = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); strip < nb * ns; strip += warps)
-        split_strip<false>(DenseRows{F, ldf, n, vec}, n, n_pad, a, b, digit_scale, rscale, rinv, s, out, bnorm2, strip,
-                           lane, tr);
+    for (int u = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < nb * ns * PIECES; u += warps)
+        split_strip<false, NR>(DenseRows{F, ldf, n, vec}, n, n_pad, a, b, digit_scale, rscale, rinv, s, out,
+                               NR == 32 ? bnorm2 : nullptr, u / PIECES, lane, tr, nullptr, u % PIECES * NR);
     if (red) {
         tr = warp_sum_f(tr);
         if (lane == 0) atomicAdd(red, (double)tr);
@@ -210,13 +219,14 @@ __global__ void __launch_bounds__(256) split_kernel(const double* __restrict__ F
 
 // The splits of many matrices in one launch (a batch's f_0 for every
 // instance): strip u of the launch belongs to the job with the largest
-// strip0 <= u; the warp that takes a job's first strip also clears its
+// strip0 <= u; the warp that takes a job's first piece also clears its
 // four-double reduction slot.
 __global__ void __launch_bounds__(256) split_group_kernel(const SplitJob* __restrict__ jobs, int njobs,
                                                           int total_strips) {
     const int lane = threadIdx.x & 31;
     const int warps = gridDim.x * (blockDim.x >> 5);
-    for (int u = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < total_strips; u += warps) {
+    for (int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < total_strips * kSplitPieces; q += warps) {
+        const int u = q / kSplitPieces, piece = q % kSplitPieces;
         int lo = 0, hi = njobs - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -227,11 +237,12 @@ __global__ void __launch_bounds__(256) split_group_kernel(const SplitJob* __rest
         }
         const SplitJob& J = jobs[lo];
         const int strip = u - J.strip0;
-        if (strip == 0 && J.zero4 && lane < 4) J.zero4[lane] = 0.0;
+        if (strip == 0 && piece == 0 && J.zero4 && lane < 4) J.zero4[lane] = 0.0;
         const bool vec = (J.ldf & 1) == 0 && ((uintptr_t)J.F & 15) == 0;
         float tr = 0.f;
-        split_strip<false>(DenseRows{J.F, J.ldf, J.n, vec}, J.n, J.n_pad, df{J.a_h, J.a_l}, df{J.b_h, J.b_l},
-                           J.digit_scale, J.rscale, 1.f / J.rscale, J.s, J.out, nullptr, strip, lane, tr);
+        split_strip<false, kSplitRows>(DenseRows{J.F, J.ldf, J.n, vec}, J.n, J.n_pad, df{J.a_h, J.a_l},
+                                       df{J.b_h, J.b_l}, J.digit_scale, J.rscale, 1.f / J.rscale, J.s, J.out, nullptr,
+                                       strip, lane, tr, nullptr, piece * kSplitRows);
     }
 }
 
@@ -248,7 +259,7 @@ __global__ void __launch_bounds__(256) split_pool_kernel(const double* __restric
     const float rinv = 1.f / rscale;
     float tr = 0.f;
     for (int strip = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); strip < nb * ns; strip += warps)
-        split_strip<true>(DenseRows{F, ldf, n, vec}, n, n_pad, a, b, digit_scale, rscale, rinv, s, pool, bnorm2, strip,
+        split_strip<true, 32>(DenseRows{F, ldf, n, vec}, n, n_pad, a, b, digit_scale, rscale, rinv, s, pool, bnorm2, strip,
                           lane, tr, pidx);
 }
 
@@ -268,7 +279,7 @@ __global__ void __launch_bounds__(256) split_csr_pool_kernel(const int64_t* __re
     const CsrRows rows{ptr, col, val, n, rowbuf[warp]};
     float tr = 0.f;
     for (int q = blockIdx.x * (blockDim.x >> 5) + warp; q < nstrips; q += warps)
-        split_strip<true>(rows, n, n_pad, a, b, digit_scale, rscale, rinv, s, pool, bnorm2, strips[q], lane, tr,
+        split_strip<true, 32>(rows, n, n_pad, a, b, digit_scale, rscale, rinv, s, pool, bnorm2, strips[q], lane, tr,
                           pidx);
 }
 
@@ -648,7 +659,7 @@ int make_split_job(const double* F, int64_t ldf, int n, int n_pad, double a, dou
 int launch_split_group(const SplitJob* jobs, int njobs, int total_strips, cudaStream_t stream) {
     if (njobs <= 0 || total_strips <= 0) return PURIFY_OK;
     if (!jobs) return PURIFY_ERR_INVALID_ARG;
-    int64_t blocks = ((int64_t)total_strips + 7) / 8;  // 8 warps per CTA, one strip each
+    int64_t blocks = ((int64_t)total_strips * kSplitPieces + 7) / 8;  // 8 warps per CTA, one piece each
     if (blocks > 152 * 8) blocks = 152 * 8;
     split_group_kernel<<<(unsigned)blocks, 256, 0, stream>>>(jobs, njobs, total_strips);
     PURIFY_CUDA_TRY(cudaGetLastError());
@@ -694,10 +705,12 @@ int launch_split(const double* F, int64_t ldf, int n, int n_pad, double a, doubl
         rbits > 8)
         return PURIFY_ERR_INVALID_ARG;
     const int64_t strips = (int64_t)(n_pad / 32) * (n_pad / 128);
-    int64_t blocks = (strips + 7) / 8;  // 8 warps per CTA, one 32 x 128 strip each
+    const int64_t pieces = bnorm2 ? strips : strips * kSplitPieces;
+    int64_t blocks = (pieces + 7) / 8;  // 8 warps per CTA, one 32 x 128 strip or piece each
     if (blocks > 152 * 8) blocks = 152 * 8;
-    split_kernel<<<(unsigned)blocks, 256, 0, stream>>>(F, ldf, n, n_pad, to_df(a), to_df(b), ldexpf(1.f, 8 - e),
-                                                        ldexpf(1.f, rbits), s, out, red, bnorm2);
+    auto kernel = bnorm2 ? split_kernel<32> : split_kernel<kSplitRows>;
+    kernel<<<(unsigned)blocks, 256, 0, stream>>>(F, ldf, n, n_pad, to_df(a), to_df(b), ldexpf(1.f, 8 - e),
+                                                 ldexpf(1.f, rbits), s, out, red, bnorm2);
     PURIFY_CUDA_TRY(cudaGetLastError());
     count_launches(1);
     return PURIFY_OK;
