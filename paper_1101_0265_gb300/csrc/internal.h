@@ -73,6 +73,10 @@ int launch_lanczos_f64(const double* F, int64_t n, int k, double* scratch, cudaS
                        const CsrF* csr = nullptr);
 int64_t lanczos_scratch_doubles(int64_t n, int k);
 // Offsets of the a / bsq arrays inside the Lanczos scratch.
+// the word whose upper half is set when a device wait of the steps ran out (the
+// coefficients are then meaningless), directly before a and bsq
+inline int64_t lanczos_flag_offset(int64_t n) { return 3 * n; }
+int lanczos_flag_status(double flag);
 inline int64_t lanczos_a_offset(int64_t n) { return 3 * n + 1; }
 inline int64_t lanczos_bsq_offset(int64_t n, int k) { return 3 * n + 1 + k; }
 

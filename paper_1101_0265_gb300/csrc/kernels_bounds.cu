@@ -6,6 +6,7 @@
 // warp per row reads the row with coalesced 8-byte loads.
 #include <cuda.h>
 
+#include "grid_sync.cuh"
 #include "internal.h"
 
 #include <cmath>
@@ -313,6 +314,130 @@ lanczos_shift_kernel(double* __restrict__ vprev, double* __restrict__ v, const d
     }
 }
 
+// block_sum256 of the first 256 threads' values, called by every thread of a
+// larger block (whose other warps stay off the float64 pipe: a warp's
+// instruction takes 16 cycles there, whatever its lanes do).
+__device__ double block_sum_first256(double v) {
+    __shared__ double ws[8];
+    __shared__ double total;
+    if (threadIdx.x < 256) v = warp_sum(v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0 && threadIdx.x < 256) ws[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int q = 0; q < 8; ++q) t += ws[q];
+        total = t;
+    }
+    __syncthreads();
+    return total;
+}
+
+// All k Lanczos steps of a dense F in one cooperative launch (one block per
+// SM), in the arithmetic and the order of the kernels above: the same
+// coefficients bit for bit.  Per step
+//   1. w = F v - b_{j-1} v_prev, one warp per row, and the row's share of w . v;
+//      v in shared memory;                                              barrier
+//   2. the first vec_blocks(n) blocks: a_j, w -= a_j v, pb[block];       barrier
+//   3. every block: b_j^2, its own copy of the next v = w / b_j.
+// A warp keeps eight loads in flight; for large n, 1 is bound by the float64 pipe
+// (2 FMAs per clock and SM).
+constexpr int kCoopMaxN = 8192;
+constexpr int kCoopThreads = 1024;
+
+__global__ void __launch_bounds__(kCoopThreads)
+lanczos_coop_kernel(const double* __restrict__ F, int n, int k, int vb, double* v0, double* w0, double* w1, double* dots,
+                    double* pb, double* a, double* bsq, GridSync* sync) {
+    extern __shared__ double sv[];  // v | v_prev, n each
+    __shared__ double bi[2];
+    double* v = sv;
+    double* vp = sv + n;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int groups = (n + LZ_ROWS - 1) / LZ_ROWS;
+    unsigned int round = 0;
+    for (int i = tid; i < n; i += kCoopThreads) {
+        v[i] = v0[i];
+        vp[i] = 0.0;
+    }
+    __syncthreads();
+    double b = 0.0;
+    for (int j = 0; j < k; ++j) {
+        // (w alternates: a block may still read the previous one in 3)
+        double* w = (j & 1) ? w1 : w0;
+        for (int i = warp * gridDim.x + blockIdx.x; i < n; i += (kCoopThreads / 32) * gridDim.x) {
+            const double* row = F + (int64_t)i * n;
+            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+            int c = lane;
+            for (; c + 224 < n; c += 256) {
+                double f[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) f[q] = row[c + 32 * q];
+#pragma unroll
+                for (int q = 0; q < 8; q += 4) {
+                    s0 = fma(f[q], v[c + 32 * q], s0);
+                    s1 = fma(f[q + 1], v[c + 32 * q + 32], s1);
+                    s2 = fma(f[q + 2], v[c + 32 * q + 64], s2);
+                    s3 = fma(f[q + 3], v[c + 32 * q + 96], s3);
+                }
+            }
+            for (; c + 96 < n; c += 128) {
+                s0 = fma(row[c], v[c], s0);
+                s1 = fma(row[c + 32], v[c + 32], s1);
+                s2 = fma(row[c + 64], v[c + 64], s2);
+                s3 = fma(row[c + 96], v[c + 96], s3);
+            }
+            for (; c < n; c += 32) s0 = fma(row[c], v[c], s0);
+            const double s = warp_sum((s0 + s1) + (s2 + s3));
+            if (lane == 0) {
+                const double wi = s - b * vp[i];
+                w[i] = wi;
+                dots[i] = wi * v[i];
+            }
+        }
+        grid_barrier(sync, round);
+        if ((int)blockIdx.x < vb) {
+            // the rows' shares group by group, then the groups as sum_parts256 takes them
+            double p = 0.0;
+            if (tid < 256)
+                for (int g = tid; g < groups; g += 256) {
+                    double t = 0.0;
+#pragma unroll
+                    for (int r = 0; r < LZ_ROWS; ++r)
+                        if (LZ_ROWS * g + r < n) t += __ldcg(dots + LZ_ROWS * g + r);
+                    p += t;
+                }
+            const double aj = block_sum_first256(p);
+            if (blockIdx.x == 0 && tid == 0) a[j] = aj;
+            double s = 0.0;
+            for (int i = blockIdx.x * 256 + tid; i < n && tid < 256; i += vb * 256) {
+                const double wi = __ldcg(w + i) - aj * v[i];
+                w[i] = wi;
+                s += wi * wi;
+            }
+            s = block_sum_first256(s);
+            if (tid == 0) pb[blockIdx.x] = s;
+        }
+        grid_barrier(sync, round);
+        double p = 0.0;
+        if (tid < 256)
+            for (int q = tid; q < vb; q += 256) p += __ldcg(pb + q);
+        const double b2 = block_sum_first256(p);
+        if (blockIdx.x == 0 && tid == 0) bsq[j] = b2;
+        if (tid == 0) {  // (one warp: the square root and the division are long)
+            bi[0] = sqrt(b2);
+            bi[1] = bi[0] > 0.0 ? 1.0 / bi[0] : 0.0;
+        }
+        __syncthreads();
+        b = bi[0];
+        const double inv = bi[1];
+        for (int i = tid; i < n; i += kCoopThreads) {
+            vp[i] = v[i];
+            v[i] = __ldcg(w + i) * inv;
+        }
+        __syncthreads();
+    }
+}
+
 unsigned vec_blocks(int64_t n) {
     int64_t b = (n + 255) / 256;
     if (b > kVecBlocksMax) b = kVecBlocksMax;
@@ -350,7 +475,7 @@ int launch_gershgorin_csr_f64(const CsrF& F, int64_t n, double* lohi, double* sc
 }
 
 int64_t lanczos_scratch_doubles(int64_t n, int k) {
-    return 3 * n + 1 + 2 * (int64_t)k + (n + LZ_ROWS - 1) / LZ_ROWS + kVecBlocksMax;
+    return 3 * n + 1 + 2 * (int64_t)k + (n + LZ_ROWS - 1) / LZ_ROWS + kVecBlocksMax + (n <= kCoopMaxN ? n : 0);
 }
 
 int launch_lanczos_f64(const double* F, int64_t n, int k, double* scratch, cudaStream_t s, const CsrF* csr) {
@@ -367,6 +492,34 @@ int launch_lanczos_f64(const double* F, int64_t n, int k, double* scratch, cudaS
     const unsigned vb = vec_blocks(n);
     lanczos_start_kernel<<<vb, 256, 0, s>>>(v, vprev, n, pb);
     scale_by_norm_kernel<<<vb, 256, 0, s>>>(v, n, pb, (int)vb, qn);
+    GridSync* sync = (GridSync*)qn;
+    PURIFY_CUDA_TRY(cudaMemsetAsync(sync, 0, sizeof(GridSync), s));
+    // Measured, purify_set_hamiltonian with 16 steps (three launches a step -> one
+    // launch): n = 130 414 -> 275 us, n = 1000 501 -> 367, n = 4096 1102 -> 925, n =
+    // 8192 3213 -> 2738.  Larger v and v_prev would not fit in shared memory.
+    if (!csr && n <= kCoopMaxN) {
+        int dev = 0, sms = 0;
+        PURIFY_CUDA_TRY(cudaGetDevice(&dev));
+        PURIFY_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        PURIFY_CUDA_TRY(cudaFuncSetAttribute((const void*)lanczos_coop_kernel,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * kCoopMaxN));
+        int ni = (int)n, vbi = (int)vb;
+        double* dots = pb + kVecBlocksMax;
+        // (a row per warp: small matrices leave SMs out, and the barrier is shorter)
+        const int need = (int)((n + 15) / 16), grid = need < sms ? (need > vbi ? need : vbi) : sms;
+        if (vbi <= sms) {
+            void* args[] = {(void*)&F, &ni, &k, &vbi, &v, &w, &vprev, &dots, &pb, &a, &bsq, &sync};
+            const cudaError_t e = cudaLaunchCooperativeKernel((const void*)lanczos_coop_kernel, dim3(grid), dim3(kCoopThreads),
+                                                              args, 16 * (size_t)n, s);
+            if (e == cudaSuccess) {
+                count_launches(3);
+                return PURIFY_OK;
+            }
+            if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported)
+                return cuda_status(e, "cudaLaunchCooperativeKernel");
+            cudaGetLastError();  // not all blocks fit at once: step by step
+        }
+    }
     for (int j = 0; j < k; ++j) {
         if (csr)
             lanczos_matvec_csr_kernel<<<(unsigned)rows, 32 * LZ_ROWS, 0, s>>>(

@@ -323,6 +323,12 @@ void tridiag_eig_full(const double* a, const double* b, int m, std::vector<doubl
     }
 }
 
+int lanczos_flag_status(double flag) {
+    uint64_t bits;
+    std::memcpy(&bits, &flag, sizeof(bits));
+    return bits >> 32 ? PURIFY_ERR_DEVICE_TIMEOUT : PURIFY_OK;
+}
+
 int host_bounds_from_lanczos(const double* a, const double* bsq, int k, double g_lo, double g_hi,
                              double* lo, double* hi) {
     // Truncate at an exact breakdown (b_j == 0: invariant subspace found).
@@ -624,13 +630,12 @@ static int finish_set(purify_t h, int64_t n, int64_t nocc, double mu, const puri
             double* ls = h->scratch + 2;  // Gershgorin partials are consumed already
             PURIFY_TRY(launch_lanczos_f64(h->F, n, k, ls, h->stream, csr ? &cf : nullptr));
             PURIFY_CUDA_TRY(cudaMemcpyAsync(g, lohi, sizeof(g), cudaMemcpyDeviceToHost, h->stream));
-            std::vector<double> a(k), bsq(k);
-            PURIFY_CUDA_TRY(cudaMemcpyAsync(a.data(), ls + lanczos_a_offset(n), sizeof(double) * k,
+            std::vector<double> ab(1 + 2 * (size_t)k);  // flag | a | bsq
+            PURIFY_CUDA_TRY(cudaMemcpyAsync(ab.data(), ls + lanczos_flag_offset(n), sizeof(double) * ab.size(),
                                             cudaMemcpyDeviceToHost, h->stream));
-            PURIFY_CUDA_TRY(cudaMemcpyAsync(bsq.data(), ls + lanczos_bsq_offset(n, k),
-                                            sizeof(double) * k, cudaMemcpyDeviceToHost, h->stream));
             PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
-            PURIFY_TRY(host_bounds_from_lanczos(a.data(), bsq.data(), k, g[0], g[1], &lo, &hi));
+            PURIFY_TRY(lanczos_flag_status(ab[0]));
+            PURIFY_TRY(host_bounds_from_lanczos(&ab[1], &ab[1 + k], k, g[0], g[1], &lo, &hi));
         } else {
             PURIFY_CUDA_TRY(cudaMemcpyAsync(g, lohi, sizeof(g), cudaMemcpyDeviceToHost, h->stream));
             PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
@@ -1379,8 +1384,11 @@ int purify_k_lanczos_f64(const double* F, int64_t n, int k, double* a, double* b
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(bsq.data(), scratch + lanczos_bsq_offset(n, k), sizeof(double) * k,
                                 cudaMemcpyDeviceToHost, s);
+        double flag = 0.0;
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&flag, scratch + lanczos_flag_offset(n), sizeof(double), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) r = cuda_status(e, "lanczos copy-out");
+        r = e != cudaSuccess ? cuda_status(e, "lanczos copy-out") : lanczos_flag_status(flag);
     }
     cudaFree(scratch);
     if (r != PURIFY_OK) return r;
