@@ -27,6 +27,7 @@
 
 #include "digits_tc.h"
 #include "f64_digits.h"
+#include "grid_sync.cuh"
 #include "internal.h"
 #include "mixed.h"
 
@@ -175,6 +176,169 @@ dot_kernel(const double* __restrict__ a, const double* __restrict__ b, int64_t n
     if (threadIdx.x == 0) parts[blockIdx.x] = s;
 }
 
+// block_sum256 of the first 256 threads' values, called by every thread of a
+// larger block (whose other warps stay off the float64 pipe: a warp's
+// instruction takes 16 cycles there, whatever its lanes do).
+__device__ double block_sum_first256(double v) {
+    __shared__ double ws[8];
+    __shared__ double total;
+    if (threadIdx.x < 256) v = warp_sum_d(v);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0 && threadIdx.x < 256) ws[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int q = 0; q < 8; ++q) t += ws[q];
+        total = t;
+    }
+    __syncthreads();
+    return total;
+}
+
+// Sum of partials that other blocks of the running launch wrote.
+__device__ double sum_parts_cg(const double* p, int count) {
+    double s = 0.0;
+    if (threadIdx.x < 256)
+        for (int q = threadIdx.x; q < count; q += 256) s += __ldcg(p + q);
+    return block_sum_first256(s);
+}
+
+// The k Lanczos steps of both filters (side 0: X^4 (I - X), side 1: X (I - X)^4)
+// in one cooperative launch, one block per SM, in the arithmetic and the order of
+// the kernels above: the same coefficients bit for bit.  Both sides' vectors
+// meet each row of X together, one warp per row.  Per step five matvecs (the input
+// vectors in shared memory; a barrier after each), then the two vector passes on
+// the first vec_grid(n) blocks of each side.  ROWS: the block keeps its rows of X
+// in shared memory for all steps (n up to about 1850 on 152 SMs).  The matvecs are
+// bound by the float64 pipe (2 FMAs per clock and SM: 7.8 us at n = 1500), small
+// ones by the barriers.  Measured, purify_estimate_gap with 40 steps (a launch per
+// matvec and vector pass, the sides one after the other -> here): n = 333 7.9 -> 3.4 ms,
+// n = 1500 11.4 -> 6.7 ms, n = 2500 18.3 -> 15.1 ms (the kernel itself 1.06, 2.5 and 7.1).
+constexpr int kFilterMaxN = 8192;
+constexpr int kFilterThreads = 512;
+constexpr size_t kFilterSmem = 225 * 1024;
+
+struct FilterLanczos {
+    const double* X;
+    int n, k, vb;
+    double* V[2];    // (k + 1) x n Lanczos bases, row 0 given
+    double* t[2][2]; // matvec results, alternating
+    double* w[2];
+    double* pa[2];
+    double* pb[2];
+    double* ab[2];   // a[k] | bsq[k]
+    GridSync* sync;
+};
+
+template <bool ROWS>
+__global__ void __launch_bounds__(kFilterThreads) filter_lanczos_kernel(const FilterLanczos L) {
+    extern __shared__ double sv[];  // the current vectors of both sides
+    __shared__ double bs[2], invs[2];
+    const int n = L.n, k = L.k, vb = L.vb, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int side = (int)blockIdx.x < vb ? 0 : 1;              // of the vector passes
+    const int vblock = (int)blockIdx.x - side * vb;             // (no block of them when >= vb)
+    unsigned int round = 0;
+    constexpr int kWarps = kFilterThreads / 32;
+    double* rows = sv + 2 * (size_t)n;
+    if (ROWS) {
+        int slot = warp;
+        for (int i = warp * gridDim.x + blockIdx.x; i < n; i += kWarps * gridDim.x, slot += kWarps)
+            for (int c = lane; c < n; c += 32) rows[(size_t)slot * n + c] = L.X[(size_t)i * n + c];
+    }
+    double b = 0.0;  // this block's side: b_{j-1}
+    for (int j = 0; j < k; ++j) {
+        if (j == 0) {
+            for (int i = tid; i < n; i += kFilterThreads) {
+                sv[i] = L.V[0][i];
+                sv[n + i] = L.V[1][i];
+            }
+        } else {
+            double b2[2];
+            b2[0] = sum_parts_cg(L.pb[0], vb);
+            b2[1] = sum_parts_cg(L.pb[1], vb);
+            if (warp < 2 && lane == 0) {  // (one warp a side: square roots and divisions are long)
+                const double bq = sqrt((warp ? b2[1] : b2[0]));
+                bs[warp] = bq;
+                invs[warp] = bq > 0.0 ? 1.0 / bq : 0.0;
+                if (vblock == 0 && warp == side) L.ab[warp][k + j - 1] = (warp ? b2[1] : b2[0]);
+            }
+            __syncthreads();
+            b = bs[side];
+            const double inv[2] = {invs[0], invs[1]};
+            for (int i = tid; i < n; i += kFilterThreads) {
+                sv[i] = __ldcg(L.w[0] + i) * inv[0];
+                sv[n + i] = __ldcg(L.w[1] + i) * inv[1];
+            }
+        }
+        __syncthreads();
+        if (j > 0 && vblock < vb && tid < 256)
+            for (int i = vblock * 256 + tid; i < n; i += vb * 256) L.V[side][(size_t)j * n + i] = sv[side * n + i];
+        for (int st = 0; st <= kFilterPower; ++st) {
+            // side 0: X v, and at last v - X v; side 1: v - X v, and at last X v
+            const bool last = st == kFilterPower;
+            double* y0 = L.t[0][st & 1];
+            double* y1 = L.t[1][st & 1];
+            int slot = warp;
+            for (int i = warp * gridDim.x + blockIdx.x; i < n; i += kWarps * gridDim.x, slot += kWarps) {
+                const double* row = ROWS ? rows + (size_t)slot * n : L.X + (size_t)i * n;
+                double s0 = 0.0, s1 = 0.0;
+#pragma unroll 8
+                for (int c = lane; c < n; c += 32) {
+                    const double x = row[c];
+                    s0 = fma(x, sv[c], s0);
+                    s1 = fma(x, sv[n + c], s1);
+                }
+                s0 = warp_sum_d(s0);
+                s1 = warp_sum_d(s1);
+                if (lane < 2) {  // lane: the side
+                    const double s = lane ? s1 : s0, z = sv[(lane ? n : 0) + i];
+                    (lane ? y1 : y0)[i] = ((lane != 0) != last) ? z - s : s;
+                }
+            }
+            grid_barrier(L.sync, round);
+            if (!last) {
+                for (int i = tid; i < n; i += kFilterThreads) {
+                    sv[i] = __ldcg(y0 + i);
+                    sv[n + i] = __ldcg(y1 + i);
+                }
+                __syncthreads();
+            }
+        }
+        // w = t - b_{j-1} v_{j-1}, its share of w . v_j; then w -= a_j v_j
+        const double* t = L.t[side][kFilterPower & 1];
+        double* w = L.w[side];
+        const double* v = L.V[side] + (size_t)j * n;
+        if (vblock < vb) {
+            double s = 0.0;
+            for (int i = vblock * 256 + tid; i < n && tid < 256; i += vb * 256) {
+                const double wi = j ? fma(-b, v[i - n], __ldcg(t + i)) : __ldcg(t + i);
+                w[i] = wi;
+                s += wi * v[i];
+            }
+            s = block_sum_first256(s);
+            if (tid == 0) L.pa[side][vblock] = s;
+        }
+        grid_barrier(L.sync, round);
+        if (vblock < vb) {
+            const double a = sum_parts_cg(L.pa[side], vb);
+            if (vblock == 0 && tid == 0) L.ab[side][j] = a;
+            double s = 0.0;
+            for (int i = vblock * 256 + tid; i < n && tid < 256; i += vb * 256) {
+                const double wi = w[i] - a * v[i];
+                w[i] = wi;
+                s += wi * wi;
+            }
+            s = block_sum_first256(s);
+            if (tid == 0) L.pb[side][vblock] = s;
+        }
+        grid_barrier(L.sync, round);
+    }
+    if (vblock == 0) {
+        const double b2 = sum_parts_cg(L.pb[side], vb);
+        if (tid == 0) L.ab[side][2 * k - 1] = b2;
+    }
+}
+
 unsigned vec_grid(int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, kVecBlocks)); }
 
 // Device work space of one estimate.
@@ -187,6 +351,7 @@ struct GapWork {
     double* u = nullptr;   // Ritz vector
     double* parts = nullptr;  // 2 x kVecBlocks partials
     double* ab = nullptr;     // a[k] | bsq[k] | z[k]
+    GridSync* sync = nullptr;
 };
 
 int matvec(const double* X, int64_t n, const double* v, double alpha, double beta, const double* z, double* y,
@@ -228,19 +393,27 @@ int dot(const double* a, const double* b, int64_t n, GapWork& g, cudaStream_t s,
     return PURIFY_OK;
 }
 
-// k Lanczos steps on one filter of X; the top Ritz value, its residual norm
-// and the Ritz vector's Rayleigh quotient with X.
-int lanczos_top(const double* X, int64_t n, bool occupied, int k, GapWork& g, cudaStream_t s, double* theta,
-                double* resid, double* rq) {
+// The normalised start vector into v.
+int start_vector(double* v, int64_t n, GapWork& g, cudaStream_t s) {
+    const unsigned vb = vec_grid(n);
+    double* pb = g.parts + kVecBlocks;
+    start_kernel<<<vb, 256, 0, s>>>(v, n, pb);
+    normalize_kernel<<<vb, 256, 0, s>>>(v, n, pb, (int)vb);
+    PURIFY_CUDA_TRY(cudaGetLastError());
+    count_launches(2);
+    return PURIFY_OK;
+}
+
+// k Lanczos steps on one filter of X, launch by launch: n above kFilterMaxN,
+// where a matvec is long against a launch, and devices on which the
+// cooperative launch does not fit.
+int lanczos_steps_one(const double* X, int64_t n, bool occupied, int k, GapWork& g, cudaStream_t s) {
     const unsigned vb = vec_grid(n);
     double* pa = g.parts;
     double* pb = g.parts + kVecBlocks;
     double* a = g.ab;
     double* bsq = g.ab + k;
-    start_kernel<<<vb, 256, 0, s>>>(g.V, n, pb);
-    normalize_kernel<<<vb, 256, 0, s>>>(g.V, n, pb, (int)vb);
-    PURIFY_CUDA_TRY(cudaGetLastError());
-    count_launches(2);
+    PURIFY_TRY(start_vector(g.V, n, g, s));
     for (int j = 0; j < k; ++j) {
         const double* v = g.V + (size_t)j * n;
         PURIFY_TRY(apply_filter(X, n, occupied, v, g, s));
@@ -251,6 +424,59 @@ int lanczos_top(const double* X, int64_t n, bool occupied, int k, GapWork& g, cu
         PURIFY_CUDA_TRY(cudaGetLastError());
         count_launches(3);
     }
+    return PURIFY_OK;
+}
+
+// The same for both filters in one launch (work spaces g[0]: occupied, g[1]:
+// unoccupied); *done = false when it does not apply.
+int lanczos_steps_both(const double* X, int64_t n, int k, GapWork (&g)[2], cudaStream_t s, bool* done) {
+    *done = false;
+    int dev = 0, sms = 0;
+    PURIFY_CUDA_TRY(cudaGetDevice(&dev));
+    PURIFY_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    FilterLanczos L;
+    L.vb = (int)vec_grid(n);
+    if (n > kFilterMaxN || 2 * L.vb > sms) return PURIFY_OK;
+    L.X = X;
+    L.n = (int)n;
+    L.k = k;
+    for (int q = 0; q < 2; ++q) {
+        PURIFY_TRY(start_vector(g[q].V, n, g[q], s));
+        L.V[q] = g[q].V;
+        L.t[q][0] = g[q].t1;
+        L.t[q][1] = g[q].t2;
+        L.w[q] = g[q].w;
+        L.pa[q] = g[q].parts;
+        L.pb[q] = g[q].parts + kVecBlocks;
+        L.ab[q] = g[q].ab;
+    }
+    L.sync = g[0].sync;
+    PURIFY_CUDA_TRY(cudaMemsetAsync(L.sync, 0, sizeof(GridSync), s));
+    const int grid = (int)std::min<int64_t>(sms, std::max<int64_t>(2 * L.vb, (n + 3) / 4));
+    const size_t vec_bytes = 16 * (size_t)n, row_bytes = 8 * (size_t)n * (size_t)((n + grid - 1) / grid);
+    const bool rows = vec_bytes + row_bytes <= kFilterSmem;
+    const void* kernel = rows ? (const void*)filter_lanczos_kernel<true> : (const void*)filter_lanczos_kernel<false>;
+    PURIFY_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFilterSmem));
+    void* args[] = {&L};
+    const cudaError_t e = cudaLaunchCooperativeKernel(kernel, dim3(grid), dim3(kFilterThreads), args,
+                                                      vec_bytes + (rows ? row_bytes : 0), s);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        return PURIFY_OK;
+    }
+    PURIFY_CUDA_TRY(e);
+    count_launches(1);
+    *done = true;
+    return PURIFY_OK;
+}
+
+// After k Lanczos steps on a filter of X (g.V, g.ab): the top Ritz value, its
+// residual norm and the Ritz vector's Rayleigh quotient with X.
+int lanczos_top(const double* X, int64_t n, int k, GapWork& g, cudaStream_t s, double* theta, double* resid,
+                double* rq) {
+    const unsigned vb = vec_grid(n);
+    double* a = g.ab;
+    double* bsq = g.ab + k;
     std::vector<double> ha(k), hb(k);
     PURIFY_CUDA_TRY(cudaMemcpyAsync(ha.data(), a, sizeof(double) * k, cudaMemcpyDeviceToHost, s));
     PURIFY_CUDA_TRY(cudaMemcpyAsync(hb.data(), bsq, sizeof(double) * k, cudaMemcpyDeviceToHost, s));
@@ -341,7 +567,7 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
     }
     std::vector<int> branches;
     const double thr = 1.0 / (4.0 * std::sqrt((double)n));
-    GapWork g;
+    GapWork g[2];  // occupied and unoccupied side
     std::vector<void*> allocs;
     auto alloc = [&](double** p, size_t count) {
         if (cudaMalloc(p, sizeof(double) * count) != cudaSuccess) return false;
@@ -351,10 +577,30 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
     auto release = [&]() {
         for (void* p : allocs) cudaFree(p);
     };
-    if (!alloc(&g.V, (size_t)(k + 1) * n) || !alloc(&g.t, n) || !alloc(&g.w, n) || !alloc(&g.t1, n) ||
-        !alloc(&g.t2, n) || !alloc(&g.u, n) || !alloc(&g.parts, 2 * kVecBlocks) || !alloc(&g.ab, 3 * (size_t)k)) {
+    // one allocation: per side the basis, six vectors, the partials, the
+    // coefficients; then the barrier's words
+    const size_t side_doubles = (size_t)(k + 1) * n + 5 * (size_t)n + 2 * kVecBlocks + 3 * (size_t)k;
+    double* work = nullptr;
+    if (!alloc(&work, 2 * side_doubles + 1)) {
         release();
         return PURIFY_ERR_OOM;
+    }
+    for (int q = 0; q < 2; ++q) {
+        double* p = work + q * side_doubles;
+        auto take = [&p](size_t count) {
+            double* r = p;
+            p += count;
+            return r;
+        };
+        g[q].V = take((size_t)(k + 1) * n);
+        g[q].t = take(n);
+        g[q].w = take(n);
+        g[q].t1 = take(n);
+        g[q].t2 = take(n);
+        g[q].u = take(n);
+        g[q].parts = take(2 * kVecBlocks);
+        g[q].ab = take(3 * (size_t)k);
+        g[q].sync = (GridSync*)(work + 2 * side_doubles);
     }
     h->f64_on = false;
     if (!mixed) {
@@ -419,8 +665,20 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
             // X_i satisfies the switch condition: filtered Lanczos on it
             const double* Xs = Xf[(i + 1) & 1];
             double th_o, r_o, rq_o, th_u, r_u, rq_u;
-            r = lanczos_top(Xs, n, true, k, g, s, &th_o, &r_o, &rq_o);
-            if (r == PURIFY_OK) r = lanczos_top(Xs, n, false, k, g, s, &th_u, &r_u, &rq_u);
+            bool both = false;
+            r = lanczos_steps_both(Xs, n, k, g, s, &both);
+            if (r == PURIFY_OK && !both) r = lanczos_steps_one(Xs, n, true, k, g[0], s);
+            if (r == PURIFY_OK && !both) r = lanczos_steps_one(Xs, n, false, k, g[1], s);
+            if (r == PURIFY_OK && both) {
+                GridSync sy{};
+                if (cudaMemcpyAsync(&sy, g[0].sync, sizeof(sy), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+                    cudaStreamSynchronize(s) != cudaSuccess)
+                    r = PURIFY_ERR_CUDA;
+                else if (sy.failed)
+                    r = PURIFY_ERR_DEVICE_TIMEOUT;
+            }
+            if (r == PURIFY_OK) r = lanczos_top(Xs, n, k, g[0], s, &th_o, &r_o, &rq_o);
+            if (r == PURIFY_OK) r = lanczos_top(Xs, n, k, g[1], s, &th_u, &r_u, &rq_u);
             if (r != PURIFY_OK) {
                 release();
                 return r;
