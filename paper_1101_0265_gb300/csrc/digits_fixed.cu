@@ -39,8 +39,11 @@ int fill_digit_params(const DigitStep& st, DigitGemmParams* p, CUtensorMap* ma, 
 
 namespace {
 
-constexpr int kThreads = 64 + 32 * 8;
-constexpr int kMaxRegs = 168;
+// 16 epilogue warps, each 32 rows x 32 columns of a tile: with 8 an emptying of the
+// accumulators waits on its own arithmetic (two warps per scheduler)
+constexpr int kEpi = 16;
+constexpr int kThreads = 64 + 32 * kEpi;
+constexpr int kMaxRegs = 96;  // 18 warps: five on a sub-partition of 16384 registers
 
 struct FixedLaunch {
     CUtensorMap map_a, map_b;
@@ -117,7 +120,7 @@ __global__ void __maxnreg__(kMaxRegs) digit_fixed_kernel(const __grid_constant__
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2 * kStages; ++i) mbar_init(smem_u32(&full_bar[i]), 1);
         mbar_init(smem_u32(tmem_full), 1);
-        mbar_init(smem_u32(tmem_empty), 8);
+        mbar_init(smem_u32(tmem_empty), kEpi);
         mbar_init(smem_u32(drain), 1);
         *abort_flag = 0;
         fence_barrier_init();
@@ -196,8 +199,8 @@ __global__ void __maxnreg__(kMaxRegs) digit_fixed_kernel(const __grid_constant__
             mbar_wait_for(smem_u32(drain), 0);
         }
     } else {
-        // epilogue warps: lane quarter warp % 4, columns 0..63 or 64..127
-        const int quarter = warp & 3, col0 = ((warp - 2) >> 2) * 64;
+        // epilogue warps: lane quarter warp % 4, the (warp - 2) / 4-th 32 columns
+        const int quarter = warp & 3, col0 = ((warp - 2) >> 2) * (TILE * 4 / kEpi);
         const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)col0;
         bool bad = false;
         for (int t = blockIdx.x, lt = 0; t < L.items; t += gridDim.x, ++lt) {
@@ -220,10 +223,10 @@ __global__ void __maxnreg__(kMaxRegs) digit_fixed_kernel(const __grid_constant__
             uint32_t r[2][32];
             tmem_issue32(taddr, r[0]);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
+            for (int q = 0; q < TILE * 4 / kEpi / 8; ++q) {
                 uint32_t(&v)[32] = r[q & 1];
                 tmem_wait32(v);
-                if (q < 7) {
+                if (q < TILE * 4 / kEpi / 8 - 1) {
                     tmem_issue32(taddr + (uint32_t)(8 * (q + 1)), r[(q + 1) & 1]);
                 } else {
                     tc_fence_before();

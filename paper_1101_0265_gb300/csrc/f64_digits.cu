@@ -38,9 +38,9 @@
 // share panels in L2; the tiles of the last, partial wave are cut evenly over
 // the grid at stage boundaries (at n = 256, three tiles on 103 CTAs).
 //
-// Measured, one step (float64 FMA kernel -> here): n = 256 281 -> 20.5 us, n =
-// 1000 1064 -> 64 us, n = 4096 57 ms -> 1.83 ms, of which the product kernel is
-// 1.56 ms: 1.95 PFLOP/s of digit pairs, the measured bf16 burst rate.  Errors of
+// Measured, one step (float64 FMA kernel -> here): n = 256 23 -> 19 us, n = 1000
+// 896 -> 61 us, n = 4096 56 ms -> 1.78 ms, of which the product kernel is about 1.5
+// ms: 2.0 PFLOP/s of digit pairs (cuBLAS bf16 burst: 1.9).  Errors of
 // one step against extended precision at n = 4096: largest 2.2e-15 -> 7e-17,
 // rms 1.8e-17 -> 2.4e-18.
 //
@@ -69,8 +69,11 @@ constexpr int kDigits = 8;
 constexpr int kStages = 3;
 constexpr int kStageBytes = 64 * 1024;
 constexpr int kBoxBytes = TILE * 128;  // 128 rows of four planes' 16-wide k-chunks
-constexpr int kThreads = 64 + 32 * 8;
-constexpr int kMaxRegs = 168;
+// 16 epilogue warps, each 32 rows x 32 columns of a tile: with 8 an emptying of the
+// accumulators waits on its own arithmetic (two warps per scheduler)
+constexpr int kEpi = 16;
+constexpr int kThreads = 64 + 32 * kEpi;
+constexpr int kMaxRegs = 96;  // 18 warps: five on a sub-partition of 16384 registers
 constexpr int kExpLimit = 400;
 // MMAs per stage, which also measure the work: a high stage is 32 columns of
 // levels 0..3, a low stage 16 columns of levels 4..8
@@ -237,7 +240,7 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2 * kStages; ++i) mbar_init(smem_u32(&full_bar[i]), 1);
         mbar_init(smem_u32(tmem_full), 1);
-        mbar_init(smem_u32(tmem_empty), 8);
+        mbar_init(smem_u32(tmem_empty), kEpi);
         mbar_init(smem_u32(drain), 1);
         *abort_flag = 0;
         fence_barrier_init();
@@ -323,8 +326,8 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
             mbar_wait_for(smem_u32(drain), 0);
         }
     } else {
-        // epilogue warps: lane quarter warp % 4, columns 0..63 or 64..127
-        const int quarter = warp & 3, col0 = ((warp - 2) >> 2) * 64;
+        // epilogue warps: lane quarter warp % 4, the (warp - 2) / 4-th 32 columns
+        const int quarter = warp & 3, col0 = ((warp - 2) >> 2) * (TILE * 4 / kEpi);
         const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)col0;
         for (int lt = 0; walk.next(g); ++lt) {
             bool ready = mbar_wait_for(smem_u32(tmem_full), (uint32_t)(lt & 1));
@@ -341,10 +344,10 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
             uint32_t r[2][32];
             tmem_issue32(taddr, r[0]);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
+            for (int q = 0; q < TILE * 4 / kEpi / 8; ++q) {
                 uint32_t(&v)[32] = r[q & 1];
                 tmem_wait32(v);
-                if (q < 7) {
+                if (q < TILE * 4 / kEpi / 8 - 1) {
                     tmem_issue32(taddr + (uint32_t)(8 * (q + 1)), r[(q + 1) & 1]);
                 } else {
                     tc_fence_before();
