@@ -81,7 +81,7 @@ extern "C" {
 /* ---- arithmetic of the matrix products -------------------------------- */
 #define PURIFY_FP64    0  /* float64: products exact to 2^-57 of the row norms on the
                              tensor cores (8 integer digit planes, 64-bit sums), or
-                             float64 FMA on the SIMT pipe for small n (< 128), n above
+                             float64 FMA on the SIMT pipe for small n (< 160), n above
                              32768, values the digits cannot hold (infinities, NaN,
                              row scales beyond 2^+-400) and too little device memory  */
 #define PURIFY_MIXED   1  /* float64 values held as integer digit planes in bf16,

@@ -26,11 +26,12 @@ def _set(pur, F, h):
     pur.set_hamiltonian(F, nocc=h.nocc, mu=0.0, lmin=h.lmin, lmax=h.lmax, homo=h.homo, lumo=h.lumo)
 
 
-# the smallest size, tile edges and remainders, the split's warp / block
-# boundary (1024), one wave of tiles (2176 = 17 x 128: 153 tiles) and beyond
-@pytest.mark.parametrize("n", [128, 129, 255, 256, 257, 640, 1023, 1024, 1025, 1153, 2177])
+# the FMA kernel's sizes and the smallest one of the digits (160), tile edges and
+# remainders, the split's row boundaries (512, 1024), one wave of tiles (2176 =
+# 17 x 128: 153 tiles) and beyond
+@pytest.mark.parametrize("n", [3, 15, 16, 17, 128, 129, 159, 160, 161, 255, 256, 257, 512, 513, 640, 1023, 1024, 1025, 1153, 2177])
 def test_one_step_against_extended_precision(P, n):
-    F, h = I.dense_hamiltonian_device(I.InstanceSpec(n=n, nocc=n // 3, gap=0.05, scheme="TC_MONO", instance=n, config=91))
+    F, h = I.dense_hamiltonian_device(I.InstanceSpec(n=n, nocc=max(1, n // 3), gap=0.05, scheme="TC_MONO", instance=n, config=91))
     with P.Purifier() as pur:
         _set(pur, F, h)
         pur.run("TC_MONO", 1e-12, 0)
