@@ -615,7 +615,7 @@ __device__ __forceinline__ void finish_pass(const uint2 (&v)[NQ], const double (
 // with conversions and the diagonal's terms on the float64 pipe).  NQ = 1
 // spreads small matrices over more SMs (n = 256: 36 blocks of 32 x 32).
 template <int NQ, bool HAS_E, bool AFFINE>
-__global__ void __launch_bounds__(256, 5)
+__global__ void __launch_bounds__(256, 4)
 f64_finish_kernel(uint2* __restrict__ T, const int* __restrict__ ea, const int* __restrict__ eb,
                   const double* __restrict__ E, double* __restrict__ C, int n, int pieces, double cP, double cE,
                   double cI, double dY, double dI, double* red, const int* __restrict__ flags) {
@@ -627,33 +627,46 @@ f64_finish_kernel(uint2* __restrict__ T, const int* __restrict__ ea, const int* 
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     double s_tr = 0.0, s_idem = 0.0;
     bool any_diag = false;
-    for (int u = blockIdx.x; u < pieces; u += gridDim.x) {
-        const int b = u / PB, c0 = (u % PB) * 8 * NQ;
-        int J = (int)((sqrtf(8.f * (float)b + 1.f) - 1.f) * 0.5f);
-        while ((J + 1) * (J + 2) / 2 <= b) ++J;
-        while (J * (J + 1) / 2 > b) --J;
-        const int I = b - J * (J + 1) / 2;
-        uint2* t = T + (size_t)((J >> 2) * ((J >> 2) + 1) / 2 + (I >> 2)) * (TILE * TILE) +
-                   (size_t)((J & 3) * 32 + c0) * TILE + (I & 3) * 32 + tx;
-        const int i = I * 32 + tx, j0 = J * 32 + c0;
-        const int ei = ea[i] - 60;
+    // a piece's place, and its entries and E, read one piece ahead
+    struct Piece {
+        int I, J, c0;
+        uint2* t;
         uint2 v[NQ];
         double e[NQ];
         int ex[NQ];
+    } cur, nxt;
+    auto fetch = [&](int u, Piece& p) {
+        const int b = u / PB;
+        p.c0 = (u % PB) * 8 * NQ;
+        int J = (int)((sqrtf(8.f * (float)b + 1.f) - 1.f) * 0.5f);
+        while ((J + 1) * (J + 2) / 2 <= b) ++J;
+        while (J * (J + 1) / 2 > b) --J;
+        p.J = J;
+        p.I = b - J * (J + 1) / 2;
+        p.t = T + (size_t)((J >> 2) * ((J >> 2) + 1) / 2 + (p.I >> 2)) * (TILE * TILE) +
+              (size_t)((J & 3) * 32 + p.c0) * TILE + (p.I & 3) * 32 + tx;
+        const int i = p.I * 32 + tx, j0 = J * 32 + p.c0;
+        const int ei = ea[i] - 60;
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
             const int c = ty + 8 * q, j = j0 + c;
-            v[q] = t[c * TILE];
-            e[q] = (HAS_E && i < n && j < n) ? E[(size_t)j * n + i] : 0.0;
-            ex[q] = ei + eb[j];
+            p.v[q] = __ldcs(p.t + c * TILE);
+            p.e[q] = (HAS_E && i < n && j < n) ? E[(size_t)j * n + i] : 0.0;
+            p.ex[q] = ei + eb[j];
         }
+    };
+    if ((int)blockIdx.x < pieces) fetch(blockIdx.x, nxt);
+    for (int u = blockIdx.x; u < pieces; u += gridDim.x) {
+        cur = nxt;
+        if (u + (int)gridDim.x < pieces) fetch(u + gridDim.x, nxt);
+        const int I = cur.I, J = cur.J, i = I * 32 + tx, j0 = J * 32 + cur.c0;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) t[(ty + 8 * q) * TILE] = make_uint2(0u, 0u);
+        for (int q = 0; q < NQ; ++q) cur.t[(ty + 8 * q) * TILE] = make_uint2(0u, 0u);
         if (I == J) {
             any_diag = true;
-            finish_pass<NQ, HAS_E, AFFINE, true>(v, e, ex, i, j0, n, C, cP, cE, cI, dY, dI, tile, s_tr, s_idem);
+            finish_pass<NQ, HAS_E, AFFINE, true>(cur.v, cur.e, cur.ex, i, j0, n, C, cP, cE, cI, dY, dI, tile, s_tr, s_idem);
         } else {
-            finish_pass<NQ, HAS_E, AFFINE, false>(v, e, ex, i, j0, n, C, cP, cE, cI, dY, dI, tile, s_tr, s_idem);
+            finish_pass<NQ, HAS_E, AFFINE, false>(cur.v, cur.e, cur.ex, i, j0, n, C, cP, cE, cI, dY, dI, tile, s_tr, s_idem);
         }
         __syncthreads();
         // the row segments (i, j0 .. j0 + 8 NQ): 8 NQ threads a row
@@ -789,7 +802,7 @@ int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, d
     PURIFY_CUDA_TRY(launch_chained(f64_digit_product_kernel, (unsigned)grid, (unsigned)kThreads, kSmemBytes, s, L));
     const int64_t nb = (n + 31) / 32, blocks = nb * (nb + 1) / 2;
     auto finish = [&](auto kernel, int64_t pieces) {
-        return launch_chained(kernel, (unsigned)std::min<int64_t>(pieces, (int64_t)f.ctas * 5), 256u, 0, s, (uint2*)f.T,
+        return launch_chained(kernel, (unsigned)std::min<int64_t>(pieces, (int64_t)f.ctas * 4), 256u, 0, s, (uint2*)f.T,
                               f.exps[a], f.exps[b], E, C, (int)n, (int)pieces, cP, cE, cI, dY, dI, red, f.flags);
     };
     auto finish_nq = [&](auto e, auto affine) {
