@@ -52,7 +52,14 @@ struct FixedLaunch {
     int* err;
     long long wait_cycles;
     int items, split_begin, ways;
+    int halves;  // 2: an item's levels 0..2 (half 0) and levels >= 3 (half 1) on two CTAs
 };
+
+// Unit u of the grid: an item, or one of its halves.
+__device__ __forceinline__ int fixed_unit(const FixedLaunch& L, int u, int& half) {
+    half = u >= L.items;
+    return half ? u - L.items : u;
+}
 
 // Work item t: a tile, or a part of a tile of the last wave; and the k-chunks
 // it sums.  Item t's share of levels >= 3 is sums.shared[t].
@@ -88,6 +95,23 @@ __device__ __forceinline__ unsigned long long pack_levels(float a0, float a1, fl
         l = ((int)(__float_as_uint(t) - kMagicBits) << 12) + (int)(__float_as_uint(r) - kMagicBits);
     }
     return (unsigned long long)(unsigned int)(h + (l >> 31)) << 32 | (unsigned int)l;
+}
+
+// The MMAs of one 32-wide k-chunk for levels 0..2 (HALF 0) or for the shared
+// accumulator of levels >= 3 (HALF 1), each accumulator's in issue_chunk's order.
+template <int S, int HALF>
+__device__ __forceinline__ void issue_half(uint32_t tmem, uint64_t da, uint64_t db, uint32_t later) {
+#pragma unroll
+    for (int p = 0; p < S; ++p)
+#pragma unroll
+        for (int q = 0; q < S - p; ++q) {
+            if ((p + q >= NUM_ACC - 1) != (HALF == 1)) continue;
+            const int a = HALF ? NUM_ACC - 1 : p + q;
+#pragma unroll
+            for (int kk = 0; kk < 2; ++kk)
+                mma_bf16(tmem + (uint32_t)(a * TILE), da + (uint64_t)plane_desc_off(p, kk),
+                         db + (uint64_t)plane_desc_off(q, kk), IDESC, (kk > 0 || p > 0 || q > NUM_ACC - 1) ? 1u : later);
+        }
 }
 
 template <int S>
@@ -130,7 +154,7 @@ __global__ void __maxnreg__(kMaxRegs) digit_fixed_kernel(const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    int ti, tj, k0, count;
+    int ti, tj, k0, count, half;
     grid_dependency_wait();
     // a step controlled on the device (uniform over the grid: written by an earlier kernel)
     const DevStep* ctl = L.prm.ctl;
@@ -141,8 +165,8 @@ __global__ void __maxnreg__(kMaxRegs) digit_fixed_kernel(const __grid_constant__
         if (lane == 0) {
             int it = 0;
             bool ok = true;
-            for (int t = blockIdx.x; ok && t < L.items; t += gridDim.x) {
-                fixed_item(L, t, ti, tj, k0, count);
+            for (int u = blockIdx.x; ok && u < L.items * L.halves; u += gridDim.x) {
+                fixed_item(L, fixed_unit(L, u, half), ti, tj, k0, count);
                 for (int c = 0; c < count; ++c, ++it) {
                     const int st = it % kStages;
                     if ((it >= kStages &&
@@ -171,8 +195,8 @@ __global__ void __maxnreg__(kMaxRegs) digit_fixed_kernel(const __grid_constant__
             const uint64_t desc_base = smem_desc(smem_u32(base));
             int it = 0;
             bool ok = true;
-            for (int t = blockIdx.x, lt = 0; ok && t < L.items; t += gridDim.x, ++lt) {
-                fixed_item(L, t, ti, tj, k0, count);
+            for (int u = blockIdx.x, lt = 0; ok && u < L.items * L.halves; u += gridDim.x, ++lt) {
+                fixed_item(L, fixed_unit(L, u, half), ti, tj, k0, count);
                 if (lt > 0 && !mbar_wait_for(smem_u32(tmem_empty), (uint32_t)((lt - 1) & 1), wait)) {
                     ok = false;
                     break;
@@ -186,7 +210,14 @@ __global__ void __maxnreg__(kMaxRegs) digit_fixed_kernel(const __grid_constant__
                     }
                     tc_fence_after();
                     const uint64_t da = desc_base + (uint64_t)((st * kStageBytes) >> 4);
-                    issue_chunk<S>(tmem, da, da + (uint64_t)((NP * PAIR_BYTES) >> 4), c > 0 ? 1u : 0u);
+                    const uint64_t db = da + (uint64_t)((NP * PAIR_BYTES) >> 4);
+                    const uint32_t later = c > 0 ? 1u : 0u;
+                    if (L.halves == 1)
+                        issue_chunk<S>(tmem, da, db, later);
+                    else if (half)
+                        issue_half<S, 1>(tmem, da, db, later);
+                    else
+                        issue_half<S, 0>(tmem, da, db, later);
                     mma_commit(smem_u32(&empty_bar[st]));
                 }
                 if (ok) mma_commit(smem_u32(tmem_full));
@@ -203,7 +234,9 @@ __global__ void __maxnreg__(kMaxRegs) digit_fixed_kernel(const __grid_constant__
         const int quarter = warp & 3, col0 = ((warp - 2) >> 2) * (TILE * 4 / kEpi);
         const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)col0;
         bool bad = false;
-        for (int t = blockIdx.x, lt = 0; t < L.items; t += gridDim.x, ++lt) {
+        for (int u = blockIdx.x, lt = 0; u < L.items * L.halves; u += gridDim.x, ++lt) {
+            const int t = fixed_unit(L, u, half);
+            const bool exact = !half, rest = NA > 3 && (half || L.halves == 1);
             fixed_item(L, t, ti, tj, k0, count);
             bool ready = mbar_wait_for(smem_u32(tmem_full), (uint32_t)(lt & 1), wait);
             if (!ready) {
@@ -238,14 +271,16 @@ __global__ void __maxnreg__(kMaxRegs) digit_fixed_kernel(const __grid_constant__
                 if (ti == tj && quarter > ((col0 + 8 * q) >> 5)) continue;
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
-                    const float a0 = __uint_as_float(v[c]), a1 = __uint_as_float(v[8 + c]);
-                    bad |= !(fabsf(a0) < 4194304.f) || (NA > 1 && !(fabsf(a1) < 32768.f));
-                    const unsigned long long u = pack_levels<NA>(a0, a1, __uint_as_float(v[16 + c]));
-                    if (part)
-                        atomicAdd(sum + (8 * q + c) * TILE, u);
-                    else
-                        sum[(8 * q + c) * TILE] = u;
-                    if (NA > 3) shared[(8 * q + c) * TILE] = __uint_as_float(v[24 + c]);
+                    if (exact) {
+                        const float a0 = __uint_as_float(v[c]), a1 = __uint_as_float(v[8 + c]);
+                        bad |= !(fabsf(a0) < 4194304.f) || (NA > 1 && !(fabsf(a1) < 32768.f));
+                        const unsigned long long x = pack_levels<NA>(a0, a1, __uint_as_float(v[16 + c]));
+                        if (part)
+                            atomicAdd(sum + (8 * q + c) * TILE, x);
+                        else
+                            sum[(8 * q + c) * TILE] = x;
+                    }
+                    if (rest) shared[(8 * q + c) * TILE] = __uint_as_float(v[24 + c]);
                 }
             }
         }
@@ -476,7 +511,13 @@ int launch_fixed(const DigitStep& st, cudaStream_t stream) {
     L.wait_cycles = st.wait_cycles;
     digit_step_split(st, tiles, &L.split_begin, &L.ways);
     L.items = L.split_begin + (tiles - L.split_begin) * L.ways;
-    const int grid = std::min(L.items, st.max_ctas);
+    // An item's halves on two CTAs while each gets one (the accumulators are
+    // independent, so their sums keep their order). Per product, whole items ->
+    // halves: n = 200 (6 items) 19.6 -> 17 us, n = 512 (40) 21.2 -> 19.0 us. With
+    // more items than half the CTAs it does not pay: half 0 takes in as many
+    // operand bytes for fewer MMAs (n = 1500, 78 items: 78 -> 91 us).
+    L.halves = S > NUM_ACC - 1 && 2 * L.items <= st.max_ctas ? 2 : 1;
+    const int grid = std::min(L.items * L.halves, st.max_ctas);
     PURIFY_TRY(prepare_digit_fixed());
     PURIFY_CUDA_TRY(launch_chained(digit_fixed_kernel<S>, (unsigned)grid, (unsigned)kThreads, fixed_smem<S>(), stream, L));
     const int nb = st.n_pad / 32, blocks = nb * (nb + 1) / 2;
