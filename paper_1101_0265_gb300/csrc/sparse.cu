@@ -65,9 +65,13 @@ __global__ void drop_blocks_kernel(unsigned long long* pat, int words, int* idx,
 constexpr int kHistBins = 1 << 16;
 constexpr double kBudgetUnits = 1099511627776.0;  // 2^40
 
+constexpr int kScanThreads = 1024;                         // bins of one scan segment
+constexpr int kScanBlocks = kHistBins / kScanThreads;
+
 struct TruncSel {
-    unsigned long long hist_fx[kHistBins];
-    unsigned int hist_cnt[kHistBins];
+    unsigned long long hist_fx[2][kHistBins];  // by pass
+    unsigned long long seg[kScanBlocks];       // mass of each segment of bins
+    unsigned int arrived[2];                   // scan blocks that have summed their segment, by pass
     unsigned long long cum_before;  // mass of the keys below the found bin
     int found, bin;                 // bin of the crossing (found = 0: none)
     int hi;                         // pass 0's bin: the key's high 16 bits
@@ -103,8 +107,7 @@ __global__ void trunc_hist_kernel(const float* __restrict__ bn2, const unsigned 
         if (!trunc_candidate(bn2, pat, words, nb, idx, budget, &key, &fx, &I, &J)) continue;
         if (pass && (int)(key >> 16) != hi) continue;
         const int bin = pass ? (int)(key & 0xFFFFu) : (int)(key >> 16);
-        if (fx) atomicAdd(&sel->hist_fx[bin], fx);
-        atomicAdd(&sel->hist_cnt[bin], 1u);
+        if (fx) atomicAdd(&sel->hist_fx[pass][bin], fx);
     }
 }
 
@@ -113,71 +116,76 @@ __device__ __forceinline__ unsigned long long sat_add(unsigned long long a, unsi
     return c < a ? ~0ull : c;
 }
 
-// One CTA of 1024 threads: the first bin whose cumulative mass (added to
-// `base`) exceeds the budget; clears the histogram for the next pass.  Warp
-// w owns bins [2048 w, 2048 w + 2048) and reads them 32 at a time
-// (coalesced): first its total, then, after an exclusive prefix of the 32
-// warp totals, its bins in order with a warp scan per 32 until the crossing.
-// Sums saturate (only sums up to the crossing matter, and those stay within
-// the budget plus one bin).
-__global__ void __launch_bounds__(1024) trunc_scan_kernel(TruncSel* sel, int pass) {
-    constexpr int kWarps = 32, kPerWarp = kHistBins / kWarps;
-    __shared__ unsigned long long wsum[kWarps];
-    __shared__ int first;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned long long base = pass ? sel->cum_before : 0ull;
+// The first bin whose cumulative mass (added to that of the keys before) exceeds
+// the budget: every block sums its segment of 1024 bins, the block that arrives
+// last finds the segment of the crossing and scans its bins. Sums saturate (only
+// sums up to the crossing matter, and those stay within the budget plus one bin).
+// One block over all bins, which also cleared them for the next pass, took 55 us
+// (a single SM's bandwidth); this takes 6 (twice a step).
+__global__ void __launch_bounds__(kScanThreads) trunc_scan_kernel(TruncSel* sel, int pass) {
+    __shared__ unsigned long long wsum[kScanThreads / 32], seg[kScanBlocks];
+    __shared__ unsigned long long seg_before;
+    __shared__ int seg_found, first;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const unsigned long long budget = (unsigned long long)kBudgetUnits;
-    const unsigned long long* fx = sel->hist_fx + warp * kPerWarp;
-    const unsigned int* cnt = sel->hist_cnt + warp * kPerWarp;
-    unsigned long long s = 0;
-#pragma unroll 8
-    for (int c = lane; c < kPerWarp; c += 32) s = sat_add(s, fx[c]);
+    unsigned long long s = sel->hist_fx[pass][blockIdx.x * kScanThreads + tid];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s = sat_add(s, __shfl_xor_sync(0xffffffffu, s, o));
     if (lane == 0) wsum[warp] = s;
-    if (threadIdx.x == 0) first = kHistBins;
     __syncthreads();
-    unsigned long long cum = base;  // base + the bins of the warps before this one
-    for (int q = 0; q < warp; ++q) cum = sat_add(cum, wsum[q]);
-    int mine = kHistBins;
-    unsigned long long before = 0;
-    for (int c0 = 0; c0 < kPerWarp; c0 += 32) {
-        const unsigned long long v = fx[c0 + lane];
-        const bool has = cnt[c0 + lane] != 0;
-        unsigned long long incl = v;  // this chunk's bins up to this lane
+    if (tid == 0) {
+        unsigned long long t = 0;
+        for (int q = 0; q < kScanThreads / 32; ++q) t = sat_add(t, wsum[q]);
+        sel->seg[blockIdx.x] = t;
+        __threadfence();
+        seg_found = atomicAdd(&sel->arrived[pass], 1u) == gridDim.x - 1 ? 0 : -1;
+    }
+    __syncthreads();
+    if (seg_found < 0) return;  // another block arrives last
+    __threadfence();
+    if (tid < kScanBlocks) seg[tid] = __ldcg(&sel->seg[tid]);
+    __syncthreads();
+    if (tid == 0) {
+        unsigned long long cum = pass ? sel->cum_before : 0ull;
+        int g = 0;
+        for (; g < kScanBlocks; ++g) {
+            const unsigned long long next = sat_add(cum, seg[g]);
+            if (next > budget) break;
+            cum = next;
+        }
+        seg_before = cum;
+        seg_found = g;
+        first = kScanThreads;
+        if (g == kScanBlocks) sel->found = 0;
+    }
+    __syncthreads();
+    const int g = seg_found;
+    if (g == kScanBlocks) return;
+    const unsigned long long v = __ldcg(&sel->hist_fx[pass][g * kScanThreads + tid]);
+    unsigned long long incl = v;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long u = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl = sat_add(incl, u);
-        }
-        unsigned long long excl = __shfl_up_sync(0xffffffffu, incl, 1);
-        if (lane == 0) excl = 0ull;
-        const unsigned m = __ballot_sync(0xffffffffu, has && sat_add(cum, incl) > budget);
-        if (m) {
-            if (lane == __ffs(m) - 1) {
-                mine = warp * kPerWarp + c0 + lane;
-                before = cum + excl;
-            }
-            break;
-        }
-        cum = sat_add(cum, __shfl_sync(0xffffffffu, incl, 31));
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl = sat_add(incl, u);
     }
-    if (mine < kHistBins) atomicMin(&first, mine);
+    if (lane == 31) wsum[warp] = incl;
+    unsigned long long excl = __shfl_up_sync(0xffffffffu, incl, 1);
+    if (lane == 0) excl = 0ull;
     __syncthreads();
-    if (mine < kHistBins && mine == first) {
+    unsigned long long cum = seg_before;
+    for (int q = 0; q < warp; ++q) cum = sat_add(cum, wsum[q]);
+    const bool over = sat_add(cum, incl) > budget;
+    if (over) atomicMin(&first, tid);
+    __syncthreads();
+    if (tid == first) {
+        const int bin = g * kScanThreads + tid;
         sel->found = 1;
-        sel->bin = mine;
-        sel->cum_before = before;
+        sel->bin = bin;
+        sel->cum_before = sat_add(cum, excl);
         if (pass == 0)
-            sel->hi = mine;
+            sel->hi = bin;
         else
-            sel->key = ((unsigned)sel->hi << 16) | (unsigned)mine;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && first == kHistBins) sel->found = 0;
-    for (int b = threadIdx.x; b < kHistBins; b += 1024) {
-        sel->hist_fx[b] = 0;
-        sel->hist_cnt[b] = 0;
+            sel->key = ((unsigned)sel->hi << 16) | (unsigned)bin;
     }
 }
 
@@ -343,7 +351,7 @@ int truncate_step(purify_ctx* h, Pattern& pat, double tau, int* idx) {
     int2* tie_dev = ms->drops + upper;
     for (int pass = 0; pass < 2; ++pass) {
         trunc_hist_kernel<<<(unsigned)grid, 256, 0, h->stream>>>(ms->bnorm2, ms->pat_dev, words, nb, budget, pass, sel);
-        trunc_scan_kernel<<<1, 1024, 0, h->stream>>>(sel, pass);
+        trunc_scan_kernel<<<kScanBlocks, kScanThreads, 0, h->stream>>>(sel, pass);
     }
     trunc_collect_kernel<<<(unsigned)grid, 256, 0, h->stream>>>(ms->bnorm2, ms->pat_dev, words, nb, budget, sel,
                                                                 ms->drops, (int)upper, tie_dev, kTieCap);
