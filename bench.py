@@ -33,7 +33,7 @@ GAPS = (1e-1, 1e-2, 1e-3, 1e-4)
 SCHEMES = ("TC_SF", "FIXED_MU_SF")
 SMS = 152                        # GB300 streaming multiprocessors
 TENSOR_FLOP_PER_CLK_SM = 8192    # dense bf16 tcgen05 rate per SM and clock (nominal)
-FP64_FLOP_PER_CLK_SM = 4         # two float64 FMAs per SM and clock (nominal)
+F64_DIGIT_PAIRS = 43             # bf16 digit pairs of one float64 product (csrc/f64_digits.cu)
 # The tensor pipe's active share of one queue launch of the digit-plane
 # product (ncu sm__pipe_tensor_cycles_active of digit_gemm_kernel<32, 5, 2>:
 # one TC_SF run at n = 4096, 14 products in one launch).
@@ -713,12 +713,15 @@ def main():
                               "rate": f"{TENSOR_FLOP_PER_CLK_SM} dense bf16 flop per clock per SM "
                                       f"x {SMS} SMs (the nominal dense rate)"}}
     else:
-        achieved = acc["useful"] / acc["prod_s"] / 1e12
-        peak = SMS * FP64_FLOP_PER_CLK_SM * sm_mhz * 1e6 / 1e12
-        roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": achieved / peak, "traffic": None, "kernel": "step_f64_kernel",
-                "peak_kind": f"float64 FMA pipe: {SMS} SMs x {FP64_FLOP_PER_CLK_SM // 2} DFMA per clock x 2 "
-                             f"x the median SM clock under load ({sm_mhz:.0f} MHz)"}
+        t128 = (n + 127) // 128
+        pair_flops = t128 * (t128 + 1) / 2 * 2 * 128 * 128 * t128 * 128
+        achieved = acc["mults"] * F64_DIGIT_PAIRS * pair_flops / acc["prod_s"] / 1e12
+        peak = pk["bf16_tflops_sustained"]
+        roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                "frac": achieved / peak, "traffic": None,
+                "kernel": "float64 step: split, f64_digit_product_kernel (exact digit products on tcgen05), finish",
+                "peak_kind": f"{pk_kind} bf16 sustained", "digit_pairs": F64_DIGIT_PAIRS,
+                "useful_tflops_in_products": acc["useful"] / acc["prod_s"] / 1e12}
     line = {
         "metric": METRIC, "value": value, "unit": "matrices/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
@@ -768,7 +771,7 @@ def main():
     if ref:
         ref.close()
         line["fp64_path"] = {"value": per_step / t64, "unit": "matrices/s",
-                             "note": "same schedules through the float64 SIMT path, same GPU"}
+                             "note": "same schedules through the float64 path, same GPU"}
     elif args.precision == "fp64":
         for r in results:
             r["max_err_vs_fp64"] = 0.0
@@ -803,8 +806,8 @@ def main():
         variant("refine_fp64", args.exact_bounds, refine_fp64=1)
         variants["note"] = ("one handle in order, the same 16 purifications: exact_bounds flips how "
                             "lmin/lmax are obtained; refine_tc_6digits appends one McWeeny step at 6 digits "
-                            "on the tensor cores; refine_fp64 appends one float64 McWeeny step (two DFMA "
-                            "products) on the float64 pipe")
+                            "on the tensor cores; refine_fp64 appends one float64 McWeeny step (two "
+                            "products)")
         line["variants"] = variants
     wall["variants"] = time.perf_counter() - t_sec
     t_sec = time.perf_counter()

@@ -20,8 +20,8 @@
 // poisons the run: the finish pass writes NaN from then on.
 //
 // Measured per product of a run, host calls included (persistent kernel -> here):
-// n = 200 67 -> 20 us, n = 1101 92 -> 36 us, n = 2000 at 5 digits 130 -> 113 us, n =
-// 2500 258 -> 202 us, n = 2900 288 -> 285 us (nearly two full waves).  From two
+// n = 200 67 -> 17 us, n = 1101 92 -> 38 us, n = 2000 at 5 digits 130 -> 110 us, n =
+// 2500 258 -> 195 us, n = 2900 288 -> 275 us (nearly two full waves).  From two
 // waves on the persistent kernel's queue launches overlap one tile's epilogue
 // with the next tile's MMAs.
 #include <algorithm>

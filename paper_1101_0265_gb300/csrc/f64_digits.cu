@@ -39,7 +39,7 @@
 // the grid at stage boundaries (at n = 256, three tiles on 103 CTAs).
 //
 // Measured, one step (float64 FMA kernel -> here): n = 256 23 -> 19 us, n = 1000
-// 896 -> 61 us, n = 4096 56 ms -> 1.78 ms, of which the product kernel is about 1.5
+// 896 -> 57 us, n = 4096 56 ms -> 1.69 ms, of which the product kernel is about 1.5
 // ms: 2.0 PFLOP/s of digit pairs (cuBLAS bf16 burst: 1.9).  Errors of
 // one step against extended precision at n = 4096: largest 2.2e-15 -> 7e-17,
 // rms 1.8e-17 -> 2.4e-18.
@@ -611,8 +611,9 @@ __device__ __forceinline__ void finish_pass(const uint2 (&v)[NQ], const double (
 // red[0] += trace(Y), red[1] += ||E - P||_F^2 (HAS_E).  Reads each fixed-point
 // entry once and clears it for the next step.  At most four float64
 // operations per element of the upper triangle: at n = 4096 they take 60 us of
-// that pipe, the 40 bytes per upper element 50 us of HBM; 185 us measured (372
-// with conversions and the diagonal's terms on the float64 pipe).  NQ = 1
+// that pipe, the 40 bytes per upper element 50 us of HBM; 85 us measured (185
+// without reading a piece ahead, 372 with conversions and the diagonal's terms on
+// the float64 pipe as well).  NQ = 1
 // spreads small matrices over more SMs (n = 256: 36 blocks of 32 x 32).
 template <int NQ, bool HAS_E, bool AFFINE>
 __global__ void __launch_bounds__(256, 4)
