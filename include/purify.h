@@ -148,7 +148,7 @@ typedef struct purify_options {
                             summation order of the inexact digit levels, so results
                             stay within the mixed path's tolerance; within a process
                             one shape per kind is used, so runs are reproducible    */
-    int wait_kcycles;    /* MIXED: bound of one device-side work wait of the product
+    int wait_kcycles;    /* bound of one device-side work wait of a tensor-core product
                             kernel (a stage, tensor-memory or work-claim hand-off), in
                             thousands of SM cycles (0 = 2^31 cycles, about one second).
                             A wait that runs out stops the kernel cleanly and the call
@@ -203,10 +203,10 @@ typedef struct purify_stats_t {
     int product_launches;       /* matrix-product kernels among them (last run)          */
     int nnz_blocks;             /* block_sparse: upper 32 x 32 blocks of the result      */
     int digit_kc;               /* MIXED: k-chunk width of the last product launch        */
-    int device_flag;            /* MIXED: device error flag of the last run (0 = none;
-                                   bits 1, 2, 4, 16: a TMA-producer, MMA, epilogue or
-                                   work-claim wait gave up; bit 8: a tile's k-chunk
-                                   count and bitmask disagreed)                         */
+    int device_flag;            /* device error flag of the last run (0 = none; bits 1,
+                                   2, 4, 16: a TMA-producer, MMA, epilogue or work-claim
+                                   wait gave up; bit 32: a wait of a float64 product;
+                                   bit 8: a tile's k-chunk count and bitmask disagreed) */
     int plane_pool_mib;         /* block_sparse: peak MiB of the pooled digit planes of
                                    the iterates (both pools; 0 otherwise)                */
     int reserved;

@@ -96,6 +96,7 @@ struct F64Product {
     CUtensorMap map_a, map_b;
     unsigned long long* T;
     int* flags;
+    long long wait_cycles;            // bound of one work wait (0: WAIT_CYCLES)
     int tiles_per_row, tiles, whole;  // whole: full waves of tiles
 };
 
@@ -239,6 +240,7 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
     uint32_t* tmem_slot = (uint32_t*)(drain + 1);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long wait = L.wait_cycles > 0 ? L.wait_cycles : WAIT_CYCLES;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2 * kStages; ++i) mbar_init(smem_u32(&full_bar[i]), 1);
@@ -268,7 +270,7 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
                 for (int c = 0; c < g.count; ++c, ++it) {
                     const int st = it % kStages;
                     if ((it >= kStages &&
-                         !mbar_wait_for(smem_u32(&empty_bar[st]), (uint32_t)(((it / kStages) & 1) ^ 1))) ||
+                         !mbar_wait_for(smem_u32(&empty_bar[st]), (uint32_t)(((it / kStages) & 1) ^ 1), wait)) ||
                         *abort_flag) {
                         ok = false;
                         break;
@@ -299,14 +301,14 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
             int it = 0, lt = 0;
             bool ok = true;
             for (; ok && walk.next(g); ++lt) {
-                if (lt > 0 && !mbar_wait_for(smem_u32(tmem_empty), (uint32_t)((lt - 1) & 1))) {
+                if (lt > 0 && !mbar_wait_for(smem_u32(tmem_empty), (uint32_t)((lt - 1) & 1), wait)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 for (int c = 0; c < g.count; ++c, ++it) {
                     const int st = it % kStages;
-                    if (!mbar_wait_for(smem_u32(&full_bar[st]), (uint32_t)((it / kStages) & 1))) {
+                    if (!mbar_wait_for(smem_u32(&full_bar[st]), (uint32_t)((it / kStages) & 1), wait)) {
                         ok = false;
                         break;
                     }
@@ -333,7 +335,7 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
         const int quarter = warp & 3, col0 = ((warp - 2) >> 2) * (TILE * 4 / kEpi);
         const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)col0;
         for (int lt = 0; walk.next(g); ++lt) {
-            bool ready = mbar_wait_for(smem_u32(tmem_full), (uint32_t)(lt & 1));
+            bool ready = mbar_wait_for(smem_u32(tmem_full), (uint32_t)(lt & 1), wait);
             if (!ready) {
                 atomicOr(L.flags + 1, ERR_F64_WAIT);
                 *abort_flag = 1;
@@ -721,7 +723,7 @@ int ensure_planes(F64Digits& f, int b) {
 
 bool f64d_wanted(int64_t n) { return n >= kF64DigitsMinN && n <= kF64DigitsMaxN; }
 
-bool f64d_begin(F64Digits& f, int64_t n, int operands, cudaStream_t s, int* err) {
+bool f64d_begin(F64Digits& f, int64_t n, int operands, long long wait_cycles, cudaStream_t s, int* err) {
     *err = PURIFY_OK;
     if (!f64d_wanted(n)) return false;
     const int n_pad = pad128(n);
@@ -747,6 +749,7 @@ bool f64d_begin(F64Digits& f, int64_t n, int operands, cudaStream_t s, int* err)
     const int r = ready();
     f.held[0] = f.held[1] = nullptr;
     f.step = 0;
+    f.wait_cycles = wait_cycles;
     if (r == PURIFY_OK) return true;
     f64d_free(f);
     if (r == PURIFY_ERR_OOM)
@@ -772,6 +775,7 @@ static int split_into(F64Digits& f, int b, const double* X, int64_t n, cudaStrea
 
 int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, double* C, int64_t n, double cP,
               double cE, double cI, double dY, double dI, double* red, cudaStream_t s) {
+    f.clean = false;  // until a check has found every step so far complete
     auto place = [&](const double* X, const double* other, int* b) -> int {
         for (int q = 0; q < 2; ++q)
             if (f.held[q] == X) {
@@ -792,6 +796,7 @@ int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, d
     PURIFY_TRY(make_quad_map(&L.map_b, f.planes[b], f.n_pad));
     L.T = f.T;
     L.flags = f.flags;
+    L.wait_cycles = f.wait_cycles;
     L.tiles_per_row = f.n_pad / TILE;
     L.tiles = (int)upper_tiles(L.tiles_per_row);
     int grid = f.ctas;
@@ -823,11 +828,14 @@ int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, d
     return PURIFY_OK;
 }
 
-int f64d_check(F64Digits& f, cudaStream_t s, int* redo_from) {
+int f64d_check(F64Digits& f, cudaStream_t s, int* redo_from, int* wait_flag) {
     int v[2] = {0, 0};
     *redo_from = -1;
+    *wait_flag = 0;
+    f.clean = false;
     PURIFY_CUDA_TRY(cudaMemcpyAsync(v, f.flags, sizeof(v), cudaMemcpyDeviceToHost, s));
     PURIFY_CUDA_TRY(cudaStreamSynchronize(s));
+    *wait_flag = v[1];
     if (v[1]) return PURIFY_ERR_DEVICE_TIMEOUT;
     *redo_from = v[0] - 1;
     f.clean = v[0] == 0;

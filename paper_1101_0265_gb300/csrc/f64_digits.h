@@ -15,10 +15,11 @@ struct F64Digits {
     __nv_bfloat16* planes[2] = {nullptr, nullptr};
     int* exps[2] = {nullptr, nullptr};  // row exponents of planes[b]
     unsigned long long* T = nullptr;    // fixed-point product, upper 128 x 128 tiles; zero between steps
-    bool clean = false;                 // T is zero (the last run ended well)
+    bool clean = false;                 // T is zero (every step queued so far was checked and ended well)
     int* flags = nullptr;  // [0] the step (from 1) whose operand left the digits' range; [1] a wait that ran out
     const double* held[2] = {nullptr, nullptr};  // the run's matrix whose digits planes[b] hold
     int step = 0;                                // steps queued since f64d_begin
+    long long wait_cycles = 0;                   // bound of the products' work waits (0: the default)
 };
 
 // Sizes that take the digit products (see f64_digits.cu).
@@ -28,7 +29,7 @@ bool f64d_wanted(int64_t n);
 // cleared state for a new run's steps.  False when the size does not want
 // them or the device has no room (the caller then takes launch_step_f64); *err
 // receives other failures.
-bool f64d_begin(F64Digits& f, int64_t n, int operands, cudaStream_t s, int* err);
+bool f64d_begin(F64Digits& f, int64_t n, int operands, long long wait_cycles, cudaStream_t s, int* err);
 
 // launch_step_f64 by exact digit products (red[2] is not reduced); A, B and E are
 // exactly symmetric.
@@ -37,8 +38,9 @@ int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, d
 
 // Synchronises; the step (from 0) from which the run has to be taken up
 // again with launch_step_f64 because its operand cannot be held (-1: none;
-// that step and all later ones have written nothing).
-int f64d_check(F64Digits& f, cudaStream_t s, int* redo_from);
+// that step and all later ones have written nothing).  PURIFY_ERR_DEVICE_TIMEOUT
+// and *wait_flag != 0 when a device wait ran out.
+int f64d_check(F64Digits& f, cudaStream_t s, int* redo_from, int* wait_flag);
 
 void f64d_free(F64Digits& f);
 

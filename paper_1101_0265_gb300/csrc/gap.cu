@@ -645,7 +645,7 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
             if (digits) {
                 int redo = -1;
                 r = f64d_step(*h->f64, Xi, Xi, Xi, Xf[i & 1], n, cP, cE, 0.0, 1.0, 0.0, red, s);
-                if (r == PURIFY_OK) r = f64d_check(*h->f64, s, &redo);
+                if (r == PURIFY_OK) r = check_f64(h, &redo);
                 if (r == PURIFY_OK && redo >= 0) digits = false;  // X_i does not fit in digits
             }
             if (!digits) r = launch_step_f64(Xi, Xi, Xi, Xf[i & 1], n, cP, cE, 0.0, 1.0, 0.0, red, s);

@@ -196,6 +196,8 @@ int ensure_dense_F(purify_ctx* h);
 // as for f64d_begin.  Where the size or the device's memory does not allow
 // them, f64_on stays false and the steps take the float64 FMA kernel.
 int begin_f64(purify_ctx* h, int operands);
+// f64d_check of the handle's products; a wait that ran out goes to st.device_flag.
+int check_f64(purify_ctx* h, int* redo_from);
 // Give the buffers of the float64 digit products back to the device.
 bool release_f64(purify_ctx* h);
 // The current F as CSR (csr_valid) for the bounds and the block-sparse split.

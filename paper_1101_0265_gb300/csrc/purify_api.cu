@@ -375,8 +375,15 @@ int purify::begin_f64(purify_ctx* h, int operands) {
     if (!h->f64) h->f64 = new (std::nothrow) F64Digits();
     if (!h->f64) return PURIFY_ERR_OOM;
     int err = PURIFY_OK;
-    h->f64_on = f64d_begin(*h->f64, h->n, operands, h->stream, &err);
+    h->f64_on = f64d_begin(*h->f64, h->n, operands, 1000ll * h->opt.wait_kcycles, h->stream, &err);
     return err;
+}
+
+int purify::check_f64(purify_ctx* h, int* redo_from) {
+    int flag = 0;
+    const int r = f64d_check(*h->f64, h->stream, redo_from, &flag);
+    if (flag) h->st.device_flag = flag;
+    return r;
 }
 
 bool purify::release_f64(purify_ctx* h) {
@@ -866,7 +873,7 @@ static int refine_f64(purify_ctx* h, int R) {
     PURIFY_TRY(r);
     if (digits) {
         int redo = -1;
-        PURIFY_TRY(f64d_check(*h->f64, h->stream, &redo));
+        PURIFY_TRY(check_f64(h, &redo));
         if (redo >= 0) {  // from the refinement step that could not be finished; its input is intact
             const int r0 = redo / 2;
             x = h->cur ^ (r0 & 1);
@@ -1085,7 +1092,7 @@ static int run_fp64(purify_ctx* h, int scheme, double tol, int max_iter, double 
         h->f64_on = false;
         PURIFY_TRY(r);
         int redo = -1;
-        PURIFY_TRY(f64d_check(*h->f64, h->stream, &redo));
+        PURIFY_TRY(check_f64(h, &redo));
         if (redo < 0) {
             S = S1;
             return PURIFY_OK;
