@@ -83,7 +83,7 @@ extern "C" {
                              tensor cores (8 integer digit planes, 64-bit sums), or
                              float64 FMA on the SIMT pipe for small n (< 160), n above
                              32768, values the digits cannot hold (infinities, NaN,
-                             row scales beyond 2^+-400) and too little device memory  */
+                             row scales above 2^400) and too little device memory     */
 #define PURIFY_MIXED   1  /* float64 values held as integer digit planes in bf16,
                              multiplied exactly on the tcgen05 tensor cores with
                              fp32 accumulation in tensor memory, recombined in

@@ -46,9 +46,11 @@
 //
 // A step is three launches: split (unless the operand's digits are still at
 // hand), product, finish.  An operand with an infinity, a NaN or a row scale
-// outside 2^+-400 sets flags[0]: the kernels of that step and of all later
-// ones leave at once, and the caller takes the run up again from that step
-// with the float64 FMA kernel, which carries such values as before.
+// above 2^400 sets flags[0]: the kernels of that step and of all later ones leave
+// at once, and the caller goes on with the float64 FMA kernel, which carries such
+// values (a run from its start, the gap estimate and the refinement from that
+// step).  Rows that underflow (a decoupled unoccupied orbital squared step after
+// step) keep the scale 2^-400.
 #include "f64_digits.h"
 
 #include <algorithm>
@@ -455,13 +457,9 @@ f64_split_kernel(const double* __restrict__ X, int n, int n_pad, __nv_bfloat16* 
         }
     };
     unsigned int top = 0;  // the largest high word: sign off, exponent and 20 leading bits
-    unsigned int low = 0;  // the low words' bits
     for_row(n, [&](int, double (&x)[4]) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            top = max(top, (unsigned int)__double2hiint(x[c]) & 0x7fffffffu);
-            low |= (unsigned int)__double2loint(x[c]);
-        }
+        for (int c = 0; c < 4; ++c) top = max(top, (unsigned int)__double2hiint(x[c]) & 0x7fffffffu);
     });
     top = row_reduce<TPR>(top, [](unsigned int a, unsigned int b) { return max(a, b); });
     const int emax = (int)(top >> 20);
@@ -479,14 +477,13 @@ f64_split_kernel(const double* __restrict__ X, int n, int n_pad, __nv_bfloat16* 
     ss = row_reduce<TPR>(ss, [](float a, float b) { return a + b; });
     // the smallest k with 4^k > ss (raised by the truncation and the sum's rounding)
     const int lg = (int)(__float_as_uint(ss * 1.01f) >> 23) - 127;
-    const int e = emax == 0 ? 0 : emax - 1023 + ((lg + 2) >> 1);
-    // outside the digits' range: not finite, denormal, or a scale beyond 2^+-400
-    if (emax == 0) {
-        if ((top | low) != 0) atomicCAS(flags, 0, step + 1);
-    } else if (t == 0 && (emax == 2047 || e > kExpLimit || e < -kExpLimit)) {
-        atomicCAS(flags, 0, step + 1);
+    // a row of zeros or below 2^-400 keeps the exponent -400: what its digits leave
+    // out is below 2^-457
+    const int e = max(emax == 0 ? -kExpLimit : emax - 1023 + ((lg + 2) >> 1), -kExpLimit);
+    if (t == 0) {
+        if (emax == 2047 || e > kExpLimit) atomicCAS(flags, 0, step + 1);  // digits cannot hold it
+        exps[i] = e;
     }
-    if (t == 0) exps[i] = e;
     for_row(n_pad, [&](int j0, double (&x)[4]) {
         uint32_t w[kDigits][2];
 #pragma unroll

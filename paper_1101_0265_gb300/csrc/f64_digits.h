@@ -36,9 +36,9 @@ bool f64d_begin(F64Digits& f, int64_t n, int operands, long long wait_cycles, cu
 int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, double* C, int64_t n, double cP,
               double cE, double cI, double dY, double dI, double* red, cudaStream_t s);
 
-// Synchronises; the step (from 0) from which the run has to be taken up
-// again with launch_step_f64 because its operand cannot be held (-1: none;
-// that step and all later ones have written nothing).  PURIFY_ERR_DEVICE_TIMEOUT
+// Synchronises; the step (from 0) whose operand cannot be held, so that it has
+// to be taken with launch_step_f64 (-1: none; that step and all later ones
+// have written nothing).  PURIFY_ERR_DEVICE_TIMEOUT
 // and *wait_flag != 0 when a device wait ran out.
 int f64d_check(F64Digits& f, cudaStream_t s, int* redo_from, int* wait_flag);
 

@@ -1069,8 +1069,7 @@ static int run_fp64_steps(purify_ctx* h, int scheme, double tol, int max_iter, d
 
 // The float64 recursion: its products on the tensor cores (f64_digits.cu),
 // and, when an operand there cannot be held in digits (not finite, or a row
-// scale outside 2^+-400), the whole recursion again with the float64 FMA
-// kernel.  The buffers that either way needs come first.
+// scale above 2^400), the whole recursion again with the float64 FMA kernel.  The buffers that either way needs come first.
 static int run_fp64(purify_ctx* h, int scheme, double tol, int max_iter, double mu, Schedule& S,
                     bool trace_rule, int* iters_out, std::vector<double>& red_host) {
     PURIFY_TRY(ensure_work(h));
