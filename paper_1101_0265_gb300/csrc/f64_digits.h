@@ -17,6 +17,7 @@ struct F64Digits {
     unsigned long long* T = nullptr;    // fixed-point product, upper 128 x 128 tiles; zero between steps
     bool clean = false;                 // T is zero (every step queued so far was checked and ended well)
     int* flags = nullptr;  // [0] the step (from 1) whose operand left the digits' range; [1] a wait that ran out
+    void* rows = nullptr;  // row scales for f64d_test_entries
     const double* held[2] = {nullptr, nullptr};  // the run's matrix whose digits planes[b] hold
     int step = 0;                                // steps queued since f64d_begin
     long long wait_cycles = 0;                   // bound of the products' work waits (0: the default)
@@ -35,6 +36,11 @@ bool f64d_begin(F64Digits& f, int64_t n, int operands, long long wait_cycles, cu
 // exactly symmetric.
 int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, double* C, int64_t n, double cP,
               double cE, double cI, double dY, double dI, double* red, cudaStream_t s);
+
+// Queue a test of the run's result D (F: the run's Hamiltonian): where an entry of
+// a product of its rows would be known worse from digits than from a chain of
+// FMAs, f64d_check reports it as a step that cannot be held.
+int f64d_test_entries(F64Digits& f, const double* D, const double* F, int64_t n, cudaStream_t s);
 
 // Synchronises; the step (from 0) whose operand cannot be held, so that it has
 // to be taken with launch_step_f64 (-1: none; that step and all later ones

@@ -893,6 +893,18 @@ static int refine_f64(purify_ctx* h, int R) {
     return PURIFY_OK;
 }
 
+// The end of a run of float64 steps: the reductions' read-back, and beside it
+// the test of what digits leave of the density's small entries.
+static int end_fp64_steps(purify_ctx* h, size_t doubles, std::vector<double>& red_host) {
+    PURIFY_CUDA_TRY(cudaEventRecord(h->e1, h->stream));
+    if (h->f64_on) PURIFY_TRY(f64d_test_entries(*h->f64, h->X[h->cur], h->F, h->n, h->stream));
+    red_host.assign(doubles, 0.0);
+    PURIFY_CUDA_TRY(cudaMemcpyAsync(red_host.data(), h->red, sizeof(double) * red_host.size(), cudaMemcpyDeviceToHost,
+                                    h->stream));
+    PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
+    return PURIFY_OK;
+}
+
 static int run_fp64_steps(purify_ctx* h, int scheme, double tol, int max_iter, double mu, Schedule& S,
                           bool trace_rule, int* iters_out, std::vector<double>& red_host) {
     const int64_t n = h->n;
@@ -950,11 +962,7 @@ static int run_fp64_steps(purify_ctx* h, int scheme, double tol, int max_iter, d
             }
             h->cur = xs;
         }
-        PURIFY_CUDA_TRY(cudaEventRecord(h->e1, h->stream));
-        red_host.assign(4 * (size_t)(ppi * m + 2), 0.0);
-        PURIFY_CUDA_TRY(cudaMemcpyAsync(red_host.data(), h->red, sizeof(double) * red_host.size(),
-                                        cudaMemcpyDeviceToHost, h->stream));
-        PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
+        PURIFY_TRY(end_fp64_steps(h, 4 * (size_t)(ppi * m + 2), red_host));
         *iters_out = m;
         return PURIFY_OK;
     }
@@ -983,11 +991,7 @@ static int run_fp64_steps(purify_ctx* h, int scheme, double tol, int max_iter, d
             }
             h->cur = xs;
         }
-        PURIFY_CUDA_TRY(cudaEventRecord(h->e1, h->stream));
-        red_host.assign(4 * (size_t)(2 * m + 2), 0.0);
-        PURIFY_CUDA_TRY(cudaMemcpyAsync(red_host.data(), h->red, sizeof(double) * red_host.size(),
-                                        cudaMemcpyDeviceToHost, h->stream));
-        PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
+        PURIFY_TRY(end_fp64_steps(h, 4 * (size_t)(2 * m + 2), red_host));
         *iters_out = m;
         return PURIFY_OK;
     }
@@ -1008,11 +1012,7 @@ static int run_fp64_steps(purify_ctx* h, int scheme, double tol, int max_iter, d
             x ^= 1;
         }
         h->cur = x;
-        PURIFY_CUDA_TRY(cudaEventRecord(h->e1, h->stream));
-        red_host.assign(4 * (size_t)slots, 0.0);
-        PURIFY_CUDA_TRY(cudaMemcpyAsync(red_host.data(), h->red, sizeof(double) * red_host.size(),
-                                        cudaMemcpyDeviceToHost, h->stream));
-        PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
+        PURIFY_TRY(end_fp64_steps(h, 4 * (size_t)slots, red_host));
         *iters_out = m;
         return PURIFY_OK;
     }
@@ -1058,18 +1058,16 @@ static int run_fp64_steps(purify_ctx* h, int scheme, double tol, int max_iter, d
     }
     S.converged = done;
     h->cur = x;
-    PURIFY_CUDA_TRY(cudaEventRecord(h->e1, h->stream));
-    red_host.assign(4 * (size_t)slots, 0.0);
-    PURIFY_CUDA_TRY(cudaMemcpyAsync(red_host.data(), h->red, sizeof(double) * red_host.size(),
-                                    cudaMemcpyDeviceToHost, h->stream));
-    PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
+    PURIFY_TRY(end_fp64_steps(h, 4 * (size_t)slots, red_host));
     *iters_out = it;
     return PURIFY_OK;
 }
 
 // The float64 recursion: its products on the tensor cores (f64_digits.cu),
 // and, when an operand there cannot be held in digits (not finite, or a row
-// scale above 2^400), the whole recursion again with the float64 FMA kernel.  The buffers that either way needs come first.
+// scale above 2^400) or the density has entries that digits know too little of
+// (f64d_test_entries), the whole recursion again with the float64 FMA kernel.
+// The buffers that either way needs come first.
 static int run_fp64(purify_ctx* h, int scheme, double tol, int max_iter, double mu, Schedule& S,
                     bool trace_rule, int* iters_out, std::vector<double>& red_host) {
     PURIFY_TRY(ensure_work(h));

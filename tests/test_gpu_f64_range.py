@@ -1,5 +1,7 @@
 """Float64 runs at the ends of what digit planes can hold: rows that underflow
-stay on the tensor cores."""
+stay on the tensor cores, and a density with entries far below their rows' norms
+(decaying or weakly coupled matrices) has them as precise as the FMA kernel gives
+them."""
 import numpy as np
 import pytest
 
@@ -65,6 +67,52 @@ def test_rows_that_underflow_stay_on_the_tensor_cores(P, block, scheme):
     ref = _fma_run(P, F, -1.0, 1.0, h.homo, h.lumo, scheme)
     assert float((D - ref).abs().max()) <= 1e-12
     assert not bool(D[:200, 200:].any())  # uncoupled stays uncoupled
+
+
+def _relative(D, ref, m):
+    """Largest relative deviation over the entries of the mask m."""
+    return float(((D - ref).abs()[m] / ref.abs()[m]).max())
+
+
+# A gapped chain of alternating bonds: the density decays by 3 every second site
+# (and is zero, up to rounding, between sites an even distance apart).
+# A run of the FMA kernel keeps every entry to n u per step relative to its own
+# terms: 14 steps x 240 x 2^-53 = 4e-13, raised along the decay; 1e-8 is far
+# above that and far below what digits of a fixed point below the row norm leave
+# (2^-58 of the norm is 1e-5 of an entry of 3e-13).
+@pytest.mark.parametrize("n", [240, 513])
+@pytest.mark.parametrize("scheme", ["TC_SF", "TC_MONO"])
+def test_decaying_density_keeps_its_small_entries(P, n, scheme):
+    n -= n % 2  # strong bonds at both ends: no state in the gap
+    t = np.where(np.arange(n - 1) % 2 == 0, 0.6, 0.2)
+    F = torch.from_numpy(np.diag(t, 1) + np.diag(t, -1)).cuda()
+    with P.Purifier() as pur:
+        pur.set_hamiltonian(F, nocc=n // 2, mu=0.0, lmin=-0.81, lmax=0.81, homo=-0.4, lumo=0.4)
+        assert pur.run(scheme, 1e-12) == P.OK
+        D = torch.from_numpy(pur.density()).cuda()
+    ref = _fma_run(P, F, -0.81, 0.81, -0.4, 0.4, scheme)
+    assert float((D - ref).abs().max()) <= 1e-12
+    i = torch.arange(n, device="cuda")
+    assert _relative(D, ref, ((i[:, None] - i[None, :]) % 2 != 0) & (ref.abs() > 1e-18)) <= 1e-8
+
+
+# two dense parts coupled by entries of 1e-10 and 1e-20
+@pytest.mark.parametrize("coupling", [1e-10, 1e-20])
+def test_weak_coupling_is_kept(P, coupling):
+    a, b = I.dense_hamiltonian(150, 70, 0.1, config=102), I.dense_hamiltonian(130, 60, 0.1, config=103)
+    C = coupling * np.random.default_rng(6).standard_normal((150, 130))
+    F = _block_diagonal(a.F, b.F)
+    F[:150, 150:] = C
+    F[150:, :150] = C.T
+    F = torch.from_numpy(F).cuda()
+    with P.Purifier() as pur:
+        pur.set_hamiltonian(F, nocc=130, mu=0.0, lmin=-1.01, lmax=1.01, homo=-0.05, lumo=0.05)
+        assert pur.run("TC_SF", 1e-12) == P.OK
+        D = torch.from_numpy(pur.density()).cuda()
+    ref = _fma_run(P, F, -1.01, 1.01, -0.05, 0.05, "TC_SF")
+    off = ref[:150, 150:]
+    # (entries that cancel are left out: below a thousandth of the largest)
+    assert _relative(D[:150, 150:], off, off.abs() > 1e-3 * off.abs().max()) <= 1e-8
 
 
 # rotated spectra of every filling stay on the tensor cores (tile and split edges)
