@@ -308,8 +308,9 @@ int run_mixed_trace(purify_ctx* h, int scheme, double tol, int max_iter, Schedul
             nb = tc_map(br, a, b);
             nbb = tc_map(br, a, bb);
         }
-        // with gap bounds the last step is known before it runs; without,
-        // every step also writes the float64 density
+        // with gap bounds the last step is known before it runs (as is the last
+        // one that max_iter allows); without, every step also writes the float64
+        // density
         const bool last_known = have_gap && std::max(nb, 1.0 - nbb) <= tol;
         DigitStep st;
         st.n = n;
@@ -325,7 +326,7 @@ int run_mixed_trace(purify_ctx* h, int scheme, double tol, int max_iter, Schedul
         st.scratch = ms->scratch;
         st.max_ctas = ms->ctas;
         const int s_next = digits(nb, nbb);
-        if (!have_gap || last_known) st.out64 = D;
+        if (!have_gap || last_known || it + 1 == max_iter) st.out64 = D;
         if (!last_known) {
             st.out = ms->Xd[x ^ 1];
             st.s_out = s_next;

@@ -101,9 +101,9 @@ __global__ void trace_sched_kernel(TraceSchedDev* c, double* red, const double* 
     }
     st.s_in = c->s_cur;
     st.s_out = last ? 0 : s_next;
-    st.write64 = (!c->have_gap || last) ? 1 : 0;
-    st.done = 0;
     const int i = c->it;
+    st.write64 = (!c->have_gap || last || i + 1 >= c->max_iter) ? 1 : 0;
+    st.done = 0;
     c->hist[kHistAlpha * c->max_iter + i] = a;
     c->hist[kHistBranch * c->max_iter + i] = br;
     c->hist[kHistBeta * c->max_iter + i] = nb;
