@@ -86,6 +86,7 @@ int ensure_mixed(purify_ctx* h, int n_pad, bool planes) {
 
 int begin_products(purify_ctx* h, int n_pad) {
     MixedState* ms = h->mixed;
+    ms->fixed_left = false;
     // [0] the product kernels' error bits, [1] a fixed-point sum out of range
     PURIFY_CUDA_TRY(cudaMemsetAsync(ms->err, 0, 2 * sizeof(int), h->stream));
     if (!digits_fixed_size(n_pad, ms->ctas)) return PURIFY_OK;
@@ -104,7 +105,17 @@ int begin_products(purify_ctx* h, int n_pad) {
     return PURIFY_OK;
 }
 
-void end_products(purify_ctx* h) { h->mixed->fixed_clean = h->mixed->fixed.shared != nullptr; }
+int end_products(purify_ctx* h) {
+    MixedState* ms = h->mixed;
+    int flags[2] = {0, 0};
+    PURIFY_CUDA_TRY(cudaMemcpyAsync(flags, ms->err, sizeof(flags), cudaMemcpyDeviceToHost, h->stream));
+    PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
+    h->st.device_flag = flags[0];
+    PURIFY_TRY(device_flag_status(flags[0]));
+    ms->fixed_left = flags[1] != 0;
+    ms->fixed_clean = ms->fixed.shared != nullptr;
+    return PURIFY_OK;
+}
 
 void attach_products(purify_ctx* h, DigitStep* st) {
     MixedState* ms = h->mixed;
@@ -112,7 +123,7 @@ void attach_products(purify_ctx* h, DigitStep* st) {
         st->partial = ms->partial;
         st->split_cnt = ms->split_cnt;
     }
-    if (ms->fixed.shared) st->fixed = &ms->fixed;
+    if (ms->fixed.shared && !ms->fixed_off) st->fixed = &ms->fixed;
     st->wait_cycles = 1000ll * h->opt.wait_kcycles;
 }
 
@@ -357,12 +368,7 @@ int run_mixed_trace(purify_ctx* h, int scheme, double tol, int max_iter, Schedul
     S.converged = done;
     h->st.digit_max = dmax;
     PURIFY_CUDA_TRY(cudaEventRecord(h->e1, h->stream));
-    int err = 0;
-    PURIFY_CUDA_TRY(cudaMemcpyAsync(&err, ms->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
-    h->st.device_flag = err;
-    if (err) return device_flag_status(err);
-    end_products(h);
+    PURIFY_TRY(end_products(h));
     if (it == 0) {
         h->st.trace = tr_prev;
         h->st.idem_err_fro = NAN;
@@ -523,14 +529,9 @@ int run_mixed_poly(purify_ctx* h, int scheme, double mu, const Schedule& S, int*
     }
     PURIFY_CUDA_TRY(cudaEventRecord(h->e1, h->stream));
     red.assign(4 * (size_t)slots, 0.0);
-    int err = 0;
     PURIFY_CUDA_TRY(cudaMemcpyAsync(red.data(), h->red, sizeof(double) * red.size(), cudaMemcpyDeviceToHost,
                                     h->stream));
-    PURIFY_CUDA_TRY(cudaMemcpyAsync(&err, ms->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
-    h->st.device_flag = err;
-    if (err) return device_flag_status(err);
-    end_products(h);
+    PURIFY_TRY(end_products(h));
     h->st.trace = m > 0 ? red[4 * (size_t)(2 * (m - 1) + 1)] : NAN;
     h->st.idem_err_fro = NAN;
     return PURIFY_OK;
@@ -978,14 +979,9 @@ int run_mixed(purify_ctx* h, int scheme, double mu, const Schedule& S, int* cur,
     }
     PURIFY_CUDA_TRY(cudaEventRecord(h->e1, h->stream));
     red.assign(4 * (size_t)slots, 0.0);
-    int err = 0;
     PURIFY_CUDA_TRY(cudaMemcpyAsync(red.data(), h->red, sizeof(double) * red.size(),
                                     cudaMemcpyDeviceToHost, h->stream));
-    PURIFY_CUDA_TRY(cudaMemcpyAsync(&err, ms->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
-    h->st.device_flag = err;
-    if (err) return device_flag_status(err);
-    end_products(h);
+    PURIFY_TRY(end_products(h));
     h->st.refine_multiplications = 2 * R;
     // statistics: trace of the result; idempotency of the last squared iterate
     const int last = m + R - 1;

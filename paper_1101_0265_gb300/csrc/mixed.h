@@ -46,6 +46,8 @@ struct MixedState {
     // fixed_clean
     FixedSums fixed;
     bool fixed_clean = false;
+    bool fixed_left = false;  // a sum of the last run left their range (its results are NaN)
+    bool fixed_off = false;   // products do without them (such a run once more)
     // block-sparse runs: per-tile k-chunk counts, then (8-byte aligned) the
     // per-tile k-chunk bitmasks, in one array of 8-byte words
     unsigned long long* kc_buf = nullptr;
@@ -103,10 +105,10 @@ struct MixedState {
 // (planes = false: the state without the dense digit planes).
 int ensure_mixed(purify_ctx* h, int n_pad, bool planes = true);
 // Start a run of single products at size n_pad: clears the device flags and
-// readies the buffers of attach_products.  end_products: the run's flags were
-// read and are clear.
+// readies the buffers of attach_products.  end_products synchronises, reads the
+// flags (st.device_flag and the status returned; fixed_left).
 int begin_products(purify_ctx* h, int n_pad);
-void end_products(purify_ctx* h);
+int end_products(purify_ctx* h);
 // The handle's product buffers and options into a step (split_k: the last
 // wave's split, or fixed-point sums where the size wants them).
 void attach_products(purify_ctx* h, DigitStep* st);

@@ -1127,61 +1127,71 @@ int purify_run(purify_t h, int scheme, double tol, int max_iter) {
     if (have_gap)
         PURIFY_TRY(build_schedule(scheme, bb.lmin, bb.lmax, mu, bb.homo, bb.lumo, tol, max_iter, S));
     PURIFY_TRY(join_in(h));
-    h->cur = -1;
     const long long launches0 = launches_so_far();
-    h->pev_used = 0;
-    h->st.product_launches = 0;
-    h->st.refine_multiplications = 0;
-    h->st.tensor_flops = 0.0;
-    h->st.digit_max = 0;
-    h->st.device_flag = 0;
-    h->hist_trace.clear();
-    h->hist_idem.clear();
+    const Schedule S0 = S;
     std::vector<double> red;
     int iters = 0;
     int r;
     bool graph_run = false;  // products replayed from a graph are not timed one by one
+    auto start_run = [&] {   // also before a run is taken up again from its start
+        h->cur = -1;
+        h->pev_used = 0;
+        h->st.product_launches = 0;
+        h->st.refine_multiplications = 0;
+        h->st.tensor_flops = 0.0;
+        h->st.digit_max = 0;
+        h->st.device_flag = 0;
+        h->hist_trace.clear();
+        h->hist_idem.clear();
+        if (h->mixed) h->mixed->d_pooled = h->mixed->fixed_left = false;
+        S = S0;
+        red.clear();
+        iters = 0;
+        graph_run = false;
+    };
+    start_run();
     if (h->opt.block_sparse && h->opt.precision != PURIFY_MIXED) return PURIFY_ERR_UNSUPPORTED;
-    if (h->mixed) h->mixed->d_pooled = false;
     const bool pooled_run = h->opt.precision == PURIFY_MIXED && h->opt.block_sparse && !trace_rule &&
                             pmm_order(scheme) != 3 && !is_asymmetric(scheme);
     if (!pooled_run) PURIFY_TRY(ensure_dense_F(h));
-    auto dispatch = [&]() -> int {
-        int r;
-        if (h->opt.precision == PURIFY_MIXED) {
-            if (trace_rule && h->opt.block_sparse) return PURIFY_ERR_UNSUPPORTED;
-            if (trace_rule) {
-                // the device-side schedule, unless the host one is asked for or
-                // the bounds already meet tol before the first step
-                const bool at_start = have_gap && std::max(S.beta0, 1.0 - S.betabar0) <= tol;
-                if (h->opt.host_schedule || at_start || max_iter == 0) {
-                    r = run_mixed_trace(h, scheme, tol, max_iter, S, &h->cur, &iters);
-                } else {
-                    r = run_mixed_trace_graph(h, scheme, tol, max_iter, S, &h->cur, &iters);
-                    graph_run = true;
-                }
-            } else if (h->opt.block_sparse && (pmm_order(scheme) == 3 || is_asymmetric(scheme))) {
-                r = PURIFY_ERR_UNSUPPORTED;
-            } else if (pmm_order(scheme) == 3 || is_asymmetric(scheme)) {
-                r = run_mixed_poly(h, scheme, mu, S, &h->cur, red);
-            } else if (h->opt.block_sparse) {
-                r = run_block_sparse(h, scheme, S, &h->cur, red);
-                if (r == PURIFY_OK && h->mixed && !h->mixed->nnzb_history.empty())
-                    h->st.nnz_blocks = h->mixed->nnzb_history.back();
-            } else {
-                r = run_mixed(h, scheme, mu, S, &h->cur, red);
-            }
-            if (r == PURIFY_OK) r = refine_f64(h, h->opt.refine_fp64);
-            if (!trace_rule) iters = (int)S.alpha.size();
-        } else {
-            r = run_fp64(h, scheme, tol, max_iter, mu, S, trace_rule, &iters, red);
+    auto mixed_steps = [&]() -> int {
+        if (trace_rule) {
+            if (h->opt.block_sparse) return PURIFY_ERR_UNSUPPORTED;
+            // the device-side schedule, unless the host one is asked for or
+            // the bounds already meet tol before the first step
+            const bool at_start = have_gap && std::max(S.beta0, 1.0 - S.betabar0) <= tol;
+            if (h->opt.host_schedule || at_start || max_iter == 0)
+                return run_mixed_trace(h, scheme, tol, max_iter, S, &h->cur, &iters);
+            const int r = run_mixed_trace_graph(h, scheme, tol, max_iter, S, &h->cur, &iters);
+            graph_run = true;
+            return r;
         }
+        if (pmm_order(scheme) == 3 || is_asymmetric(scheme))
+            return h->opt.block_sparse ? PURIFY_ERR_UNSUPPORTED : run_mixed_poly(h, scheme, mu, S, &h->cur, red);
+        if (!h->opt.block_sparse) return run_mixed(h, scheme, mu, S, &h->cur, red);
+        const int r = run_block_sparse(h, scheme, S, &h->cur, red);
+        if (r == PURIFY_OK && h->mixed && !h->mixed->nnzb_history.empty())
+            h->st.nnz_blocks = h->mixed->nnzb_history.back();
+        return r;
+    };
+    auto dispatch = [&]() -> int {
+        if (h->opt.precision != PURIFY_MIXED) return run_fp64(h, scheme, tol, max_iter, mu, S, trace_rule, &iters, red);
+        int r = mixed_steps();
+        if (r == PURIFY_OK && h->mixed && h->mixed->fixed_left) {
+            start_run();
+            h->mixed->fixed_off = true;
+            r = mixed_steps();
+            h->mixed->fixed_off = false;
+        }
+        if (r == PURIFY_OK) r = refine_f64(h, h->opt.refine_fp64);
+        if (!trace_rule) iters = (int)S.alpha.size();
         return r;
     };
     r = dispatch();
     // the float64 products' buffers of an earlier run give way to this one's
     if (r == PURIFY_ERR_OOM && release_f64(h)) {
         cudaGetLastError();
+        start_run();
         r = dispatch();
     }
     if (r != PURIFY_OK) {

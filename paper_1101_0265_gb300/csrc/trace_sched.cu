@@ -180,9 +180,11 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
     double* trF = h->red + 4 * kBlock;
     PURIFY_TRY(begin_products(h, n_pad));
     // captured steps: one block of kBlock steps and a final consume
+    const void* fixed_buf = ms->fixed_off ? nullptr : ms->fixed.levels;
     const bool key_ok = ms->tgraph && ms->tg_n == n && ms->tg_smin == smin && ms->tg_smax == smax &&
                         ms->tg_state == ms->tsched && ms->tg_red == red && ms->tg_D == h->X[0] &&
-                        ms->tg_X0 == ms->Xd[0] && ms->tg_fixed == ms->fixed.levels && ms->tg_wait == o.wait_kcycles && ms->tg_split == o.split_k;
+                        ms->tg_X0 == ms->Xd[0] && ms->tg_fixed == fixed_buf && ms->tg_wait == o.wait_kcycles &&
+                        ms->tg_split == o.split_k;
     if (!key_ok) {
         if (ms->tgraph) cudaGraphExecDestroy(ms->tgraph);
         ms->tgraph = nullptr;
@@ -232,7 +234,7 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
         ms->tg_red = red;
         ms->tg_D = h->X[0];
         ms->tg_X0 = ms->Xd[0];
-        ms->tg_fixed = ms->fixed.levels;
+        ms->tg_fixed = fixed_buf;
         ms->tg_wait = o.wait_kcycles;
         ms->tg_split = o.split_k;
     }
@@ -254,14 +256,9 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
     PURIFY_CUDA_TRY(cudaEventRecord(h->e1, h->stream));
     const int m = now.it;
     std::vector<double> hist((size_t)kHistCount * max_iter);
-    int err = 0;
     PURIFY_CUDA_TRY(cudaMemcpyAsync(hist.data(), init.hist, sizeof(double) * hist.size(), cudaMemcpyDeviceToHost,
                                     h->stream));
-    PURIFY_CUDA_TRY(cudaMemcpyAsync(&err, ms->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
-    h->st.device_flag = err;
-    if (err) return device_flag_status(err);
-    end_products(h);
+    PURIFY_TRY(end_products(h));
     S.alpha.clear();
     S.branch.clear();
     S.beta.clear();
