@@ -155,7 +155,9 @@ typedef struct purify_options {
                             kernel (a stage, tensor-memory or work-claim hand-off), in
                             thousands of SM cycles (0 = 2^31 cycles, about one second).
                             A wait that runs out stops the kernel cleanly and the call
-                            returns PURIFY_ERR_DEVICE_TIMEOUT; waits for copies and
+                            returns PURIFY_ERR_DEVICE_TIMEOUT (a grid barrier of the
+                            bound and gap estimates: the steps are then launched one
+                            by one, with the same results); waits for copies and
                             MMAs already in flight at teardown keep the full bound.
                             Short values exist to exercise failure detection; a
                             nonzero value also disables autotune                   */

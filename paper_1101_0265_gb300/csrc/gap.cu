@@ -228,6 +228,7 @@ struct FilterLanczos {
     double* pb[2];
     double* ab[2];   // a[k] | bsq[k]
     GridSync* sync;
+    long long wait;  // bound of one barrier's wait
 };
 
 template <bool ROWS>
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(kFilterThreads) filter_lanczos_kernel(const Fi
                     (lane ? y1 : y0)[i] = ((lane != 0) != last) ? z - s : s;
                 }
             }
-            grid_barrier(L.sync, round);
+            grid_barrier(L.sync, round, L.wait);
             if (!last) {
                 for (int i = tid; i < n; i += kFilterThreads) {
                     sv[i] = __ldcg(y0 + i);
@@ -318,7 +319,7 @@ __global__ void __launch_bounds__(kFilterThreads) filter_lanczos_kernel(const Fi
             s = block_sum_first256(s);
             if (tid == 0) L.pa[side][vblock] = s;
         }
-        grid_barrier(L.sync, round);
+        grid_barrier(L.sync, round, L.wait);
         if (vblock < vb) {
             const double a = sum_parts_cg(L.pa[side], vb);
             if (vblock == 0 && tid == 0) L.ab[side][j] = a;
@@ -331,7 +332,7 @@ __global__ void __launch_bounds__(kFilterThreads) filter_lanczos_kernel(const Fi
             s = block_sum_first256(s);
             if (tid == 0) L.pb[side][vblock] = s;
         }
-        grid_barrier(L.sync, round);
+        grid_barrier(L.sync, round, L.wait);
     }
     if (vblock == 0) {
         const double b2 = sum_parts_cg(L.pb[side], vb);
@@ -428,8 +429,9 @@ int lanczos_steps_one(const double* X, int64_t n, bool occupied, int k, GapWork&
 }
 
 // The same for both filters in one launch (work spaces g[0]: occupied, g[1]:
-// unoccupied); *done = false when it does not apply.
-int lanczos_steps_both(const double* X, int64_t n, int k, GapWork (&g)[2], cudaStream_t s, bool* done) {
+// unoccupied); *done = false when it does not apply or one of its waits ran out.
+int lanczos_steps_both(const double* X, int64_t n, int k, long long wait_cycles, GapWork (&g)[2], cudaStream_t s,
+                       bool* done) {
     *done = false;
     int dev = 0, sms = 0;
     PURIFY_CUDA_TRY(cudaGetDevice(&dev));
@@ -451,6 +453,7 @@ int lanczos_steps_both(const double* X, int64_t n, int k, GapWork (&g)[2], cudaS
         L.ab[q] = g[q].ab;
     }
     L.sync = g[0].sync;
+    L.wait = wait_cycles;
     PURIFY_CUDA_TRY(cudaMemsetAsync(L.sync, 0, sizeof(GridSync), s));
     const int grid = (int)std::min<int64_t>(sms, std::max<int64_t>(2 * L.vb, (n + 3) / 4));
     const size_t vec_bytes = 16 * (size_t)n, row_bytes = 8 * (size_t)n * (size_t)((n + grid - 1) / grid);
@@ -466,7 +469,10 @@ int lanczos_steps_both(const double* X, int64_t n, int k, GapWork (&g)[2], cudaS
     }
     PURIFY_CUDA_TRY(e);
     count_launches(1);
-    *done = true;
+    GridSync sy{};
+    PURIFY_CUDA_TRY(cudaMemcpyAsync(&sy, L.sync, sizeof(sy), cudaMemcpyDeviceToHost, s));
+    PURIFY_CUDA_TRY(cudaStreamSynchronize(s));
+    *done = !sy.failed;
     return PURIFY_OK;
 }
 
@@ -666,17 +672,9 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
             const double* Xs = Xf[(i + 1) & 1];
             double th_o, r_o, rq_o, th_u, r_u, rq_u;
             bool both = false;
-            r = lanczos_steps_both(Xs, n, k, g, s, &both);
+            r = lanczos_steps_both(Xs, n, k, 1000ll * h->opt.wait_kcycles, g, s, &both);
             if (r == PURIFY_OK && !both) r = lanczos_steps_one(Xs, n, true, k, g[0], s);
             if (r == PURIFY_OK && !both) r = lanczos_steps_one(Xs, n, false, k, g[1], s);
-            if (r == PURIFY_OK && both) {
-                GridSync sy{};
-                if (cudaMemcpyAsync(&sy, g[0].sync, sizeof(sy), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-                    cudaStreamSynchronize(s) != cudaSuccess)
-                    r = PURIFY_ERR_CUDA;
-                else if (sy.failed)
-                    r = PURIFY_ERR_DEVICE_TIMEOUT;
-            }
             if (r == PURIFY_OK) r = lanczos_top(Xs, n, k, g[0], s, &th_o, &r_o, &rq_o);
             if (r == PURIFY_OK) r = lanczos_top(Xs, n, k, g[1], s, &th_u, &r_u, &rq_u);
             if (r != PURIFY_OK) {

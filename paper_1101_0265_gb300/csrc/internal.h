@@ -68,15 +68,18 @@ int64_t gershgorin_scratch_doubles(int64_t n);
 // k Lanczos steps; scratch holds lanczos_scratch_doubles(n, k) doubles.
 // Writes a[0..k), bsq[0..k) (squared off-diagonals) into scratch tail; the
 // host copies them out (see purify_k_lanczos_f64).  csr set: the matvecs
-// read F from CSR storage and F (dense) is not used.
+// read F from CSR storage and F (dense) is not used.  one_launch: all steps of a
+// dense F in one cooperative launch where it fits, each of its device waits bounded
+// by wait_cycles (0: about one second); the coefficients are the same either way.
 int launch_lanczos_f64(const double* F, int64_t n, int k, double* scratch, cudaStream_t s,
-                       const CsrF* csr = nullptr);
+                       const CsrF* csr = nullptr, bool one_launch = true, long long wait_cycles = 0);
 int64_t lanczos_scratch_doubles(int64_t n, int k);
 // Offsets of the a / bsq arrays inside the Lanczos scratch.
-// the word whose upper half is set when a device wait of the steps ran out (the
-// coefficients are then meaningless), directly before a and bsq
+// the word whose upper half is set when a device wait of the one launch ran out
+// (the coefficients are then meaningless, and the steps have to be taken launch by
+// launch), directly before a and bsq
 inline int64_t lanczos_flag_offset(int64_t n) { return 3 * n; }
-int lanczos_flag_status(double flag);
+bool lanczos_gave_up(double flag);
 inline int64_t lanczos_a_offset(int64_t n) { return 3 * n + 1; }
 inline int64_t lanczos_bsq_offset(int64_t n, int k) { return 3 * n + 1 + k; }
 

@@ -347,7 +347,7 @@ constexpr int kCoopThreads = 1024;
 
 __global__ void __launch_bounds__(kCoopThreads)
 lanczos_coop_kernel(const double* __restrict__ F, int n, int k, int vb, double* v0, double* w0, double* w1, double* dots,
-                    double* pb, double* a, double* bsq, GridSync* sync) {
+                    double* pb, double* a, double* bsq, GridSync* sync, long long wait) {
     extern __shared__ double sv[];  // v | v_prev, n each
     __shared__ double bi[2];
     double* v = sv;
@@ -394,7 +394,7 @@ lanczos_coop_kernel(const double* __restrict__ F, int n, int k, int vb, double* 
                 dots[i] = wi * v[i];
             }
         }
-        grid_barrier(sync, round);
+        grid_barrier(sync, round, wait);
         if ((int)blockIdx.x < vb) {
             // the rows' shares group by group, then the groups as sum_parts256 takes them
             double p = 0.0;
@@ -417,7 +417,7 @@ lanczos_coop_kernel(const double* __restrict__ F, int n, int k, int vb, double* 
             s = block_sum_first256(s);
             if (tid == 0) pb[blockIdx.x] = s;
         }
-        grid_barrier(sync, round);
+        grid_barrier(sync, round, wait);
         double p = 0.0;
         if (tid < 256)
             for (int q = tid; q < vb; q += 256) p += __ldcg(pb + q);
@@ -478,7 +478,8 @@ int64_t lanczos_scratch_doubles(int64_t n, int k) {
     return 3 * n + 1 + 2 * (int64_t)k + (n + LZ_ROWS - 1) / LZ_ROWS + kVecBlocksMax + (n <= kCoopMaxN ? n : 0);
 }
 
-int launch_lanczos_f64(const double* F, int64_t n, int k, double* scratch, cudaStream_t s, const CsrF* csr) {
+int launch_lanczos_f64(const double* F, int64_t n, int k, double* scratch, cudaStream_t s, const CsrF* csr, bool one_launch,
+                       long long wait_cycles) {
     if (n <= 0 || k <= 0 || (!F && !csr)) return PURIFY_ERR_INVALID_ARG;
     double* vprev = scratch;
     double* v = scratch + n;
@@ -497,7 +498,7 @@ int launch_lanczos_f64(const double* F, int64_t n, int k, double* scratch, cudaS
     // Measured, purify_set_hamiltonian with 16 steps (three launches a step -> one
     // launch): n = 130 414 -> 275 us, n = 1000 501 -> 367, n = 4096 1102 -> 925, n =
     // 8192 3213 -> 2738.  Larger v and v_prev would not fit in shared memory.
-    if (!csr && n <= kCoopMaxN) {
+    if (one_launch && !csr && n <= kCoopMaxN) {
         int dev = 0, sms = 0;
         PURIFY_CUDA_TRY(cudaGetDevice(&dev));
         PURIFY_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -508,7 +509,7 @@ int launch_lanczos_f64(const double* F, int64_t n, int k, double* scratch, cudaS
         // (a row per warp: small matrices leave SMs out, and the barrier is shorter)
         const int need = (int)((n + 15) / 16), grid = need < sms ? (need > vbi ? need : vbi) : sms;
         if (vbi <= sms) {
-            void* args[] = {(void*)&F, &ni, &k, &vbi, &v, &w, &vprev, &dots, &pb, &a, &bsq, &sync};
+            void* args[] = {(void*)&F, &ni, &k, &vbi, &v, &w, &vprev, &dots, &pb, &a, &bsq, &sync, &wait_cycles};
             const cudaError_t e = cudaLaunchCooperativeKernel((const void*)lanczos_coop_kernel, dim3(grid), dim3(kCoopThreads),
                                                               args, 16 * (size_t)n, s);
             if (e == cudaSuccess) {

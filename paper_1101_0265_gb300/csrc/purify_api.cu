@@ -323,10 +323,10 @@ void tridiag_eig_full(const double* a, const double* b, int m, std::vector<doubl
     }
 }
 
-int lanczos_flag_status(double flag) {
+bool lanczos_gave_up(double flag) {
     uint64_t bits;
     std::memcpy(&bits, &flag, sizeof(bits));
-    return bits >> 32 ? PURIFY_ERR_DEVICE_TIMEOUT : PURIFY_OK;
+    return (bits >> 32) != 0;
 }
 
 int host_bounds_from_lanczos(const double* a, const double* bsq, int k, double g_lo, double g_hi,
@@ -635,13 +635,16 @@ static int finish_set(purify_t h, int64_t n, int64_t nocc, double mu, const puri
             // the Lanczos steps are queued before any result is read back, so
             // the device runs the whole estimate without a host round trip
             double* ls = h->scratch + 2;  // Gershgorin partials are consumed already
-            PURIFY_TRY(launch_lanczos_f64(h->F, n, k, ls, h->stream, csr ? &cf : nullptr));
-            PURIFY_CUDA_TRY(cudaMemcpyAsync(g, lohi, sizeof(g), cudaMemcpyDeviceToHost, h->stream));
             std::vector<double> ab(1 + 2 * (size_t)k);  // flag | a | bsq
-            PURIFY_CUDA_TRY(cudaMemcpyAsync(ab.data(), ls + lanczos_flag_offset(n), sizeof(double) * ab.size(),
-                                            cudaMemcpyDeviceToHost, h->stream));
-            PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
-            PURIFY_TRY(lanczos_flag_status(ab[0]));
+            for (bool one_launch : {true, false}) {
+                PURIFY_TRY(launch_lanczos_f64(h->F, n, k, ls, h->stream, csr ? &cf : nullptr, one_launch,
+                                              1000ll * h->opt.wait_kcycles));
+                PURIFY_CUDA_TRY(cudaMemcpyAsync(g, lohi, sizeof(g), cudaMemcpyDeviceToHost, h->stream));
+                PURIFY_CUDA_TRY(cudaMemcpyAsync(ab.data(), ls + lanczos_flag_offset(n), sizeof(double) * ab.size(),
+                                                cudaMemcpyDeviceToHost, h->stream));
+                PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
+                if (!lanczos_gave_up(ab[0])) break;
+            }
             PURIFY_TRY(host_bounds_from_lanczos(&ab[1], &ab[1 + k], k, g[0], g[1], &lo, &hi));
         } else {
             PURIFY_CUDA_TRY(cudaMemcpyAsync(g, lohi, sizeof(g), cudaMemcpyDeviceToHost, h->stream));
@@ -1390,23 +1393,23 @@ int purify_k_lanczos_f64(const double* F, int64_t n, int k, double* a, double* b
     double* scratch = nullptr;
     PURIFY_CUDA_TRY(cudaMalloc(&scratch, sizeof(double) * (size_t)lanczos_scratch_doubles(n, k)));
     cudaStream_t s = (cudaStream_t)stream;
-    int r = launch_lanczos_f64(F, n, k, scratch, s);
-    std::vector<double> bsq(k);
-    if (r == PURIFY_OK) {
-        cudaError_t e = cudaMemcpyAsync(a, scratch + lanczos_a_offset(n), sizeof(double) * k,
+    std::vector<double> ab(1 + 2 * (size_t)k);  // flag | a | bsq
+    int r = PURIFY_OK;
+    for (bool one_launch : {true, false}) {
+        r = launch_lanczos_f64(F, n, k, scratch, s, nullptr, one_launch);
+        if (r != PURIFY_OK) break;
+        cudaError_t e = cudaMemcpyAsync(ab.data(), scratch + lanczos_flag_offset(n), sizeof(double) * ab.size(),
                                         cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(bsq.data(), scratch + lanczos_bsq_offset(n, k), sizeof(double) * k,
-                                cudaMemcpyDeviceToHost, s);
-        double flag = 0.0;
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(&flag, scratch + lanczos_flag_offset(n), sizeof(double), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        r = e != cudaSuccess ? cuda_status(e, "lanczos copy-out") : lanczos_flag_status(flag);
+        if (e != cudaSuccess) r = cuda_status(e, "lanczos copy-out");
+        if (r != PURIFY_OK || !lanczos_gave_up(ab[0])) break;
     }
     cudaFree(scratch);
     if (r != PURIFY_OK) return r;
-    for (int j = 0; j < k; ++j) b[j] = std::sqrt(std::max(bsq[j], 0.0));
+    for (int j = 0; j < k; ++j) {
+        a[j] = ab[1 + (size_t)j];
+        b[j] = std::sqrt(std::max(ab[1 + (size_t)k + (size_t)j], 0.0));
+    }
     return PURIFY_OK;
 }
 

@@ -1,5 +1,6 @@
-"""Bounded device waits outside the mixed products: a wait of a float64 product
-that runs out is reported and leaves the handle usable."""
+"""Bounded device waits outside the mixed products: the float64 products'
+report a time-out and leave the handle usable, the grid barriers' lead to the
+step-by-step launches with the same coefficients."""
 import numpy as np
 import pytest
 
@@ -42,3 +43,30 @@ def test_short_waits_in_a_float64_run(P, scheme, n):
         assert pur.run(scheme, 1e-12) == P.OK
         assert pur.stats()["device_flag"] == 0
         assert np.array_equal(pur.density(), ref)
+
+
+# a barrier that gives up (blocks of another stream's kernel may hold SMs for
+# long) costs time, not the call
+@pytest.mark.parametrize("n", [130, 1000, 2500])
+def test_bounds_when_the_barrier_gives_up(P, n):
+    F, h = I.reflected_hamiltonian_device(I.InstanceSpec(n=n, nocc=n // 2, gap=0.1, scheme="TC_SF", instance=n, config=106))
+    with P.Purifier() as pur:
+        pur.set_hamiltonian(F, nocc=h.nocc)
+        a = pur.stats()
+        pur.set_options(wait_kcycles=1)
+        pur.set_hamiltonian(F, nocc=h.nocc)
+        b = pur.stats()
+    assert (a["lmin"], a["lmax"]) == (b["lmin"], b["lmax"])
+    assert b["kernel_launches"] > a["kernel_launches"]  # step by step
+
+
+# below n = 160 the float64 steps wait for nothing: only the filters' barrier does
+@pytest.mark.parametrize("n", [60, 150])
+def test_gap_when_the_barrier_gives_up(P, n):
+    F, h = I.reflected_hamiltonian_device(I.InstanceSpec(n=n, nocc=2 * n // 5, gap=0.06, scheme="TC_SF", instance=n, config=107))
+    with P.Purifier() as pur:
+        pur.set_hamiltonian(F, nocc=h.nocc, lmin=h.lmin, lmax=h.lmax)
+        ref = pur.estimate_gap()
+        pur.set_options(wait_kcycles=1)
+        assert pur.estimate_gap() == ref
+        assert h.homo <= ref[0] < ref[1] <= h.lumo
