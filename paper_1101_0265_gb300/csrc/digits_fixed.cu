@@ -555,20 +555,20 @@ bool digits_fixed_size(int n_pad, int ctas) {
 bool digits_fixed_wanted(const DigitStep& st) {
     if (!st.fixed || !st.err || st.max_ctas < 1 || st.kc_cnt || st.bnorm2 || st.a_idx) return false;
     if (st.rbits != 7 || st.s_in < 2 || st.s_in > kMaxDigitPlanes) return false;
-    return digits_fixed_size(st.n_pad, st.max_ctas);
+    const int T = st.n_pad / TILE;
+    return digits_fixed_size(st.n_pad, st.max_ctas) && T * (T + 1) / 2 <= st.fixed->tiles;
 }
 
-// Less than two waves of tiles and at most a wave of parts, two or more to a
-// split tile.
-int alloc_fixed_sums(int ctas, FixedSums* f) {
+// A tile has at most four parts; a product has less than two waves of tiles and at
+// most a wave of parts, two or more to a split tile (digit_split_plan).
+int alloc_fixed_sums(int tiles, int ctas, FixedSums* f) {
     const size_t tile = (size_t)TILE * TILE;
-    PURIFY_CUDA_TRY(cudaMalloc(&f->levels, 2 * ctas * tile * sizeof(unsigned long long)));
-    PURIFY_CUDA_TRY(cudaMalloc(&f->parts, digits_fixed_part_bytes(ctas)));
-    PURIFY_CUDA_TRY(cudaMalloc(&f->shared, 2 * ctas * tile * sizeof(float)));
+    f->parts_bytes = std::min(tiles, ctas / 2 + 1) * tile * sizeof(unsigned long long);
+    PURIFY_CUDA_TRY(cudaMalloc(&f->levels, tiles * tile * sizeof(unsigned long long)));
+    PURIFY_CUDA_TRY(cudaMalloc(&f->parts, f->parts_bytes));
+    PURIFY_CUDA_TRY(cudaMalloc(&f->shared, std::min(4 * tiles, 2 * ctas) * tile * sizeof(float)));
+    f->tiles = tiles;
     return PURIFY_OK;
-}
-size_t digits_fixed_part_bytes(int ctas) {
-    return (size_t)(ctas / 2 + 1) * TILE * TILE * sizeof(unsigned long long);
 }
 void free_fixed_sums(FixedSums* f) {
     cudaFree(f->levels);

@@ -11,11 +11,10 @@ namespace purify {
 bool digits_fixed_wanted(const DigitStep& st);
 bool digits_fixed_size(int n_pad, int ctas);
 
-// Buffers for every size of this path (70 MB on 152 SMs), their release, and the
-// bytes of FixedSums::parts.
-int alloc_fixed_sums(int ctas, FixedSums* f);
+// Buffers for products of up to `tiles` tiles (0.5 MB for one, 70 MB at the end of
+// this path's range on 152 SMs) and their release.
+int alloc_fixed_sums(int tiles, int ctas, FixedSums* f);
 void free_fixed_sums(FixedSums* f);
-size_t digits_fixed_part_bytes(int ctas);
 
 // Make that path's kernels ready (once per process; call before capturing
 // launches into a graph).

@@ -47,6 +47,8 @@ struct FixedSums {
     unsigned long long* parts = nullptr;
     float* shared = nullptr;
     int* poison = nullptr;
+    int tiles = 0;           // the most tiles of a product these buffers hold
+    size_t parts_bytes = 0;
 };
 
 // One fused step: P = A B (A, B symmetric, held as s_in digit planes each,

@@ -90,17 +90,19 @@ int begin_products(purify_ctx* h, int n_pad) {
     // [0] the product kernels' error bits, [1] a fixed-point sum out of range
     PURIFY_CUDA_TRY(cudaMemsetAsync(ms->err, 0, 2 * sizeof(int), h->stream));
     if (!digits_fixed_size(n_pad, ms->ctas)) return PURIFY_OK;
-    if (!ms->fixed.shared) {
+    const int T = n_pad / 128, tiles = T * (T + 1) / 2;
+    if (ms->fixed.tiles < tiles) {
+        free_fixed_sums(&ms->fixed);
         ms->fixed_clean = false;
-        if (alloc_fixed_sums(ms->ctas, &ms->fixed) != PURIFY_OK) {
+        ++ms->fixed_gen;
+        if (alloc_fixed_sums(tiles, ms->ctas, &ms->fixed) != PURIFY_OK) {
             free_fixed_sums(&ms->fixed);  // no room: the persistent kernel needs none
             cudaGetLastError();
             return PURIFY_OK;
         }
         ms->fixed.poison = ms->err + 1;
     }
-    if (!ms->fixed_clean)
-        PURIFY_CUDA_TRY(cudaMemsetAsync(ms->fixed.parts, 0, digits_fixed_part_bytes(ms->ctas), h->stream));
+    if (!ms->fixed_clean) PURIFY_CUDA_TRY(cudaMemsetAsync(ms->fixed.parts, 0, ms->fixed.parts_bytes, h->stream));
     ms->fixed_clean = false;
     return PURIFY_OK;
 }

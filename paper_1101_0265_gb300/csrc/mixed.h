@@ -46,6 +46,7 @@ struct MixedState {
     // fixed_clean
     FixedSums fixed;
     bool fixed_clean = false;
+    int fixed_gen = 0;        // allocations so far (a captured graph holds the addresses)
     bool fixed_left = false;  // a sum of the last run left their range (its results are NaN)
     bool fixed_off = false;   // products do without them (such a run once more)
     // block-sparse runs: per-tile k-chunk counts, then (8-byte aligned) the
@@ -70,7 +71,7 @@ struct MixedState {
     const double* tg_red = nullptr;
     const double* tg_D = nullptr;
     const void* tg_X0 = nullptr;
-    const void* tg_fixed = nullptr;
+    int tg_fixed = 0;
     // a whole run as queue launches: staging (host and device copies)
     std::vector<uint8_t> qhost;
     void* qdev = nullptr;

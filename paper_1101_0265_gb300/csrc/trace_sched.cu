@@ -180,10 +180,10 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
     double* trF = h->red + 4 * kBlock;
     PURIFY_TRY(begin_products(h, n_pad));
     // captured steps: one block of kBlock steps and a final consume
-    const void* fixed_buf = ms->fixed_off ? nullptr : ms->fixed.levels;
+    const int fixed_gen = ms->fixed_off || !ms->fixed.shared ? 0 : ms->fixed_gen;
     const bool key_ok = ms->tgraph && ms->tg_n == n && ms->tg_smin == smin && ms->tg_smax == smax &&
                         ms->tg_state == ms->tsched && ms->tg_red == red && ms->tg_D == h->X[0] &&
-                        ms->tg_X0 == ms->Xd[0] && ms->tg_fixed == fixed_buf && ms->tg_wait == o.wait_kcycles &&
+                        ms->tg_X0 == ms->Xd[0] && ms->tg_fixed == fixed_gen && ms->tg_wait == o.wait_kcycles &&
                         ms->tg_split == o.split_k;
     if (!key_ok) {
         if (ms->tgraph) cudaGraphExecDestroy(ms->tgraph);
@@ -234,7 +234,7 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
         ms->tg_red = red;
         ms->tg_D = h->X[0];
         ms->tg_X0 = ms->Xd[0];
-        ms->tg_fixed = fixed_buf;
+        ms->tg_fixed = fixed_gen;
         ms->tg_wait = o.wait_kcycles;
         ms->tg_split = o.split_k;
     }
