@@ -7,8 +7,9 @@
 
 namespace purify {
 
-// Device buffers of a handle's float64 digit products (grow only, at most
-// 2^15 rows: 39 GB).  The digits of a step's operands are kept for the run's
+// Device buffers of a handle's float64 digit products: up to kF64KeepBytes are kept
+// from run to run (and grow with the size), larger ones (at most 2^15 rows: 39
+// GB) are given back when a run has ended.  The digits of a step's operands are kept for the run's
 // next steps and forgotten at the next f64d_begin.
 struct F64Digits {
     int n_pad = 0, cap_pad = 0, ctas = 0;
@@ -48,6 +49,8 @@ int f64d_test_entries(F64Digits& f, const double* D, const double* F, int64_t n,
 // and *wait_flag != 0 when a device wait ran out.
 int f64d_check(F64Digits& f, cudaStream_t s, int* redo_from, int* wait_flag);
 
+// After a run: keep the buffers, or free them when they are large.
+void f64d_end(F64Digits& f);
 void f64d_free(F64Digits& f);
 
 }  // namespace purify

@@ -582,6 +582,7 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
     };
     auto release = [&]() {
         for (void* p : allocs) cudaFree(p);
+        end_f64(h);
     };
     // one allocation: per side the basis, six vectors, the partials, the
     // coefficients; then the barrier's words

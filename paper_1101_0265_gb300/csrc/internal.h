@@ -201,6 +201,8 @@ int ensure_dense_F(purify_ctx* h);
 int begin_f64(purify_ctx* h, int operands);
 // f64d_check of the handle's products; a wait that ran out goes to st.device_flag.
 int check_f64(purify_ctx* h, int* redo_from);
+// After the steps: large buffers go back to the device (f64d_end).
+void end_f64(purify_ctx* h);
 // Give the buffers of the float64 digit products back to the device.
 bool release_f64(purify_ctx* h);
 // The current F as CSR (csr_valid) for the bounds and the block-sparse split.

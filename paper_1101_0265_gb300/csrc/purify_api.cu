@@ -386,6 +386,10 @@ int purify::check_f64(purify_ctx* h, int* redo_from) {
     return r;
 }
 
+void purify::end_f64(purify_ctx* h) {
+    if (h->f64) f64d_end(*h->f64);
+}
+
 bool purify::release_f64(purify_ctx* h) {
     if (!h->f64 || !h->f64->cap_pad) return false;
     f64d_free(*h->f64);
@@ -1197,6 +1201,7 @@ int purify_run(purify_t h, int scheme, double tol, int max_iter) {
         start_run();
         r = dispatch();
     }
+    end_f64(h);
     if (r != PURIFY_OK) {
         h->st.status = r;
         return r;

@@ -66,3 +66,15 @@ def test_trace_rule_graphs_follow_grown_sums(P):
             pur.run("TC_MONO", 1e-4)
             out.append(pur.density())
         assert (out[0] == out[2]).all()
+
+
+def test_large_float64_workspaces_are_given_back(P):
+    n = 8192
+    F, h = I.reflected_hamiltonian_device(I.InstanceSpec(n=n, nocc=n // 2, gap=0.1, scheme="TC_SF", instance=1, config=111))
+    before = _free()
+    with P.Purifier() as pur:
+        pur.set_hamiltonian(F, nocc=h.nocc, lmin=h.lmin, lmax=h.lmax, homo=h.homo, lumo=h.lumo)
+        pur.run("TC_SF", 1e-12, 2)
+        held = before - _free()
+    # F, two iterates and the product buffer; digits and sums of this size (1.3 GiB) are given back
+    assert held <= 4 * 8 * n * n + 64 * MiB, held / MiB
