@@ -98,7 +98,7 @@ struct F64Product {
     CUtensorMap map_a, map_b;
     unsigned long long* T;
     int* flags;
-    long long wait_cycles;            // bound of one work wait (0: WAIT_CYCLES)
+    long long wait_cycles;            // bound of one work wait
     int tiles_per_row, tiles, whole;  // whole: full waves of tiles
 };
 
@@ -242,7 +242,6 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
     uint32_t* tmem_slot = (uint32_t*)(drain + 1);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long wait = L.wait_cycles > 0 ? L.wait_cycles : WAIT_CYCLES;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2 * kStages; ++i) mbar_init(smem_u32(&full_bar[i]), 1);
@@ -272,7 +271,7 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
                 for (int c = 0; c < g.count; ++c, ++it) {
                     const int st = it % kStages;
                     if ((it >= kStages &&
-                         !mbar_wait_for(smem_u32(&empty_bar[st]), (uint32_t)(((it / kStages) & 1) ^ 1), wait)) ||
+                         !mbar_wait_for(smem_u32(&empty_bar[st]), (uint32_t)(((it / kStages) & 1) ^ 1), L.wait_cycles)) ||
                         *abort_flag) {
                         ok = false;
                         break;
@@ -303,14 +302,14 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
             int it = 0, lt = 0;
             bool ok = true;
             for (; ok && walk.next(g); ++lt) {
-                if (lt > 0 && !mbar_wait_for(smem_u32(tmem_empty), (uint32_t)((lt - 1) & 1), wait)) {
+                if (lt > 0 && !mbar_wait_for(smem_u32(tmem_empty), (uint32_t)((lt - 1) & 1), L.wait_cycles)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 for (int c = 0; c < g.count; ++c, ++it) {
                     const int st = it % kStages;
-                    if (!mbar_wait_for(smem_u32(&full_bar[st]), (uint32_t)((it / kStages) & 1), wait)) {
+                    if (!mbar_wait_for(smem_u32(&full_bar[st]), (uint32_t)((it / kStages) & 1), L.wait_cycles)) {
                         ok = false;
                         break;
                     }
@@ -337,7 +336,7 @@ __global__ void __maxnreg__(kMaxRegs) f64_digit_product_kernel(const __grid_cons
         const int quarter = warp & 3, col0 = ((warp - 2) >> 2) * (TILE * 4 / kEpi);
         const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)col0;
         for (int lt = 0; walk.next(g); ++lt) {
-            bool ready = mbar_wait_for(smem_u32(tmem_full), (uint32_t)(lt & 1), wait);
+            bool ready = mbar_wait_for(smem_u32(tmem_full), (uint32_t)(lt & 1), L.wait_cycles);
             if (!ready) {
                 atomicOr(L.flags + 1, ERR_F64_WAIT);
                 *abort_flag = 1;
@@ -717,8 +716,15 @@ f64_finish_kernel(uint2* __restrict__ T, const int* __restrict__ ea, const int* 
 // The iterates need no test of their own: where one of them has small entries and
 // the density has none, those do not show in it beyond 2^-57 of the norms.
 
+// Both kernels are bound by reading D at large n and by latency at small n. They
+// work in float32 and go to float64 only for what does not fit there: all in
+// float64 they took 36 us of a call at n = 1000 and 230 us at n = 4096 (1.6 and 24.6
+// ms), now 12 and 140 us (n = 256: nothing that shows).
+
 struct RowScale {
-    double inv, diag;  // 1 / ||d_i|| (0: the row is below 2^-400 and not tested), |d_ii|
+    double inv;      // 1 / ||d_i|| (0: the row is below 2^-400 and not tested)
+    double diag;     // |d_ii|
+    float invf, diagf;
 };
 
 // One warp per row.
@@ -729,16 +735,52 @@ f64_row_scale_kernel(const double* __restrict__ D, int n, RowScale* __restrict__
     const int i = (int)blockIdx.x * 8 + (int)threadIdx.x / 32, lane = threadIdx.x & 31;
     if (i >= n) return;
     const double* row = D + (size_t)i * n;
-    double s0 = 0.0, s1 = 0.0;
-    int c = lane;
-    for (; c + 32 < n; c += 64) {
-        const double x = row[c], y = row[c + 32];
-        s0 = fma(x, x, s0);
-        s1 = fma(y, y, s1);
+    float sf = 0.f;
+    for (int c0 = 0; c0 < n; c0 += 256) {
+        float x[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) x[q] = c0 + 32 * q + lane < n ? (float)row[c0 + 32 * q + lane] : 0.f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) sf = fmaf(x[q], x[q], sf);
     }
-    if (c < n) s0 = fma(row[c], row[c], s0);
-    const double s = warp_sum_d(s0 + s1);
-    if (lane == 0) rows[i] = {s > 0x1p-800 ? rsqrt(s) : 0.0, fabs(row[i])};
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sf += __shfl_xor_sync(0xffffffffu, sf, o);
+    double s = (double)sf;
+    if (!(sf > 1e-30f && sf < 1e30f)) {
+        s = 0.0;
+        for (int c = lane; c < n; c += 32) s = fma(row[c], row[c], s);
+        s = warp_sum_d(s);
+    }
+    if (lane == 0) {
+        const double inv = s > 0x1p-800 ? rsqrt(s) : 0.0, diag = fabs(row[i]);
+        rows[i] = {inv, diag, (float)inv, (float)diag};
+    }
+}
+
+// Whether the pair (i, j) is known well enough, beyond the terms k = i and k = j
+// of the sum; false also when another pair has set the flag meanwhile.
+__device__ __noinline__ bool small_entry_passes(const double* __restrict__ D, const double* __restrict__ F, int n, int i,
+                                                int j, const RowScale& ri, const RowScale& rj, double floor,
+                                                const int* flags) {
+    const double* di = D + (size_t)i * n;
+    const double* dj = D + (size_t)j * n;
+    const double d = fabs(di[j]), w = ri.inv * rj.inv;
+    if (w == 0.0) return true;
+    if (d == 0.0) return F[(size_t)i * n + j] == 0.0;
+    double s = d * (ri.diag + rj.diag);
+    int k = i;
+    for (int c = 0; c < n && s * w < floor; c += 4) {
+        if ((c & 63) == 60 && *(const volatile int*)flags) return false;
+        double t[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {  // (the loads together)
+            const int kk = k + u < n ? k + u : k + u - n;
+            t[u] = c + u < n && kk != i && kk != j ? fabs(di[kk] * dj[kk]) : 0.0;
+        }
+        s += (t[0] + t[1]) + (t[2] + t[3]);
+        k = k + 4 < n ? k + 4 : k + 4 - n;
+    }
+    return s * w >= floor;
 }
 
 // Pairs i < j, 32 x 32 at a time, lane: j.  Nearly all pass by their terms k = i and
@@ -751,6 +793,7 @@ f64_small_entries_kernel(const double* __restrict__ D, const double* __restrict_
     grid_dependency_wait();
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const double floor = 1.0 / (16.0 * n);
+    const float quick = (float)floor * 1.0001f;
     for (int b = blockIdx.x; b < blocks; b += gridDim.x) {
         if (*(volatile int*)flags) return;
         int J = (int)((sqrtf(8.f * (float)b + 1.f) - 1.f) * 0.5f);
@@ -758,32 +801,20 @@ f64_small_entries_kernel(const double* __restrict__ D, const double* __restrict_
         while (J * (J + 1) / 2 > b) --J;
         const int I = b - J * (J + 1) / 2, j = J * 32 + tx;
         if (j >= n) continue;
-        const RowScale rj = rows[j];
+        const float inv_j = rows[j].invf, diag_j = rows[j].diagf;
+        float d[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = I * 32 + ty + 8 * q;
+            d[q] = i < j ? fabsf((float)D[(size_t)i * n + j]) : 0.f;
+        }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int i = I * 32 + ty + 8 * q;
             if (i >= j) continue;
-            const RowScale ri = rows[i];
-            const double* di = D + (size_t)i * n;
-            const double d = fabs(di[j]), w = ri.inv * rj.inv;
-            if (w == 0.0) continue;
-            if (d == 0.0) {
-                if (F[(size_t)i * n + j] != 0.0) atomicCAS(flags, 0, step + 1);
-                continue;
-            }
-            double s = d * (ri.diag + rj.diag);
-            if (s * w >= floor) continue;
-            const double* dj = D + (size_t)j * n;
-            int k = i;
-            for (int c = 0; c < n; ++c) {
-                if (k != i && k != j) s = fma(fabs(di[k]), fabs(dj[k]), s);
-                if ((c & 7) == 7) {
-                    if (s * w >= floor) break;
-                    if ((c & 63) == 63 && *(volatile int*)flags) return;
-                }
-                if (++k == n) k = 0;
-            }
-            if (!(s * w >= floor)) atomicCAS(flags, 0, step + 1);
+            const float s = d[q] * rows[i].invf * ((rows[i].diagf + diag_j) * inv_j);
+            if (s >= quick && s < 1e30f) continue;
+            if (!small_entry_passes(D, F, n, i, j, rows[i], rows[j], floor, flags)) atomicCAS(flags, 0, step + 1);
         }
     }
 }
@@ -817,6 +848,7 @@ bool f64d_begin(F64Digits& f, int64_t n, int operands, long long wait_cycles, cu
             f.cap_pad = n_pad;
             PURIFY_CUDA_TRY(cudaMalloc(&f.T, t_bytes(n_pad)));
             PURIFY_CUDA_TRY(cudaMalloc(&f.flags, 2 * sizeof(int)));
+            PURIFY_CUDA_TRY(cudaHostAlloc((void**)&f.host_flags, 2 * sizeof(int), cudaHostAllocDefault));
             PURIFY_CUDA_TRY(cudaMalloc(&f.rows, sizeof(RowScale) * n_pad));
         }
         f.n_pad = n_pad;
@@ -831,7 +863,7 @@ bool f64d_begin(F64Digits& f, int64_t n, int operands, long long wait_cycles, cu
     const int r = ready();
     f.held[0] = f.held[1] = nullptr;
     f.step = 0;
-    f.wait_cycles = wait_cycles;
+    f.wait_cycles = wait_cycles > 0 ? wait_cycles : WAIT_CYCLES;
     if (r == PURIFY_OK) return true;
     f64d_free(f);
     if (r == PURIFY_ERR_OOM)
@@ -857,7 +889,7 @@ static int split_into(F64Digits& f, int b, const double* X, int64_t n, cudaStrea
 
 int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, double* C, int64_t n, double cP,
               double cE, double cI, double dY, double dI, double* red, cudaStream_t s) {
-    f.clean = false;  // until a check has found every step so far complete
+    f.clean = f.read = false;  // until a check has found every step so far complete
     auto place = [&](const double* X, const double* other, int* b) -> int {
         for (int q = 0; q < 2; ++q)
             if (f.held[q] == X) {
@@ -921,17 +953,21 @@ int f64d_test_entries(F64Digits& f, const double* D, const double* F, int64_t n,
     return PURIFY_OK;
 }
 
-int f64d_check(F64Digits& f, cudaStream_t s, int* redo_from, int* wait_flag) {
-    int v[2] = {0, 0};
+int f64d_read(F64Digits& f, cudaStream_t s) {
+    PURIFY_CUDA_TRY(cudaMemcpyAsync(f.host_flags, f.flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    f.read = true;
+    return PURIFY_OK;
+}
+
+int f64d_check(F64Digits& f, int* redo_from, int* wait_flag) {
     *redo_from = -1;
     *wait_flag = 0;
     f.clean = false;
-    PURIFY_CUDA_TRY(cudaMemcpyAsync(v, f.flags, sizeof(v), cudaMemcpyDeviceToHost, s));
-    PURIFY_CUDA_TRY(cudaStreamSynchronize(s));
-    *wait_flag = v[1];
-    if (v[1]) return PURIFY_ERR_DEVICE_TIMEOUT;
-    *redo_from = v[0] - 1;
-    f.clean = v[0] == 0;
+    if (!f.read) return PURIFY_ERR_INTERNAL;
+    *wait_flag = f.host_flags[1];
+    if (*wait_flag) return PURIFY_ERR_DEVICE_TIMEOUT;
+    *redo_from = f.host_flags[0] - 1;
+    f.clean = f.host_flags[0] == 0;
     return PURIFY_OK;
 }
 
@@ -952,6 +988,7 @@ void f64d_free(F64Digits& f) {
     }
     cudaFree(f.T);
     cudaFree(f.flags);
+    cudaFreeHost(f.host_flags);
     cudaFree(f.rows);
     f = F64Digits();
 }

@@ -18,10 +18,12 @@ struct F64Digits {
     unsigned long long* T = nullptr;    // fixed-point product, upper 128 x 128 tiles; zero between steps
     bool clean = false;                 // T is zero (every step queued so far was checked and ended well)
     int* flags = nullptr;  // [0] the step (from 1) whose operand left the digits' range; [1] a wait that ran out
+    int* host_flags = nullptr;  // (pinned) their copy that f64d_read queued
+    bool read = false;          // ... since the last step
     void* rows = nullptr;  // row scales for f64d_test_entries
     const double* held[2] = {nullptr, nullptr};  // the run's matrix whose digits planes[b] hold
     int step = 0;                                // steps queued since f64d_begin
-    long long wait_cycles = 0;                   // bound of the products' work waits (0: the default)
+    long long wait_cycles = 0;                   // bound of the products' work waits
 };
 
 // Sizes that take the digit products (see f64_digits.cu).
@@ -43,11 +45,13 @@ int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, d
 // FMAs, f64d_check reports it as a step that cannot be held.
 int f64d_test_entries(F64Digits& f, const double* D, const double* F, int64_t n, cudaStream_t s);
 
-// Synchronises; the step (from 0) whose operand cannot be held, so that it has
-// to be taken with launch_step_f64 (-1: none; that step and all later ones
-// have written nothing).  PURIFY_ERR_DEVICE_TIMEOUT
-// and *wait_flag != 0 when a device wait ran out.
-int f64d_check(F64Digits& f, cudaStream_t s, int* redo_from, int* wait_flag);
+// Queue the read-back of the steps' flags.
+int f64d_read(F64Digits& f, cudaStream_t s);
+// After a synchronisation behind f64d_read: the step (from 0) whose operand cannot
+// be held, so that it has to be taken with launch_step_f64 (-1: none; that step
+// and all later ones have written nothing).  PURIFY_ERR_DEVICE_TIMEOUT and
+// *wait_flag != 0 when a device wait ran out.
+int f64d_check(F64Digits& f, int* redo_from, int* wait_flag);
 
 // After a run: keep the buffers, or free them when they are large.
 void f64d_end(F64Digits& f);

@@ -626,6 +626,12 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
         const int br = tr_prev > (double)h->nocc ? 1 : 0;
         const double cP = br ? 1.0 : -1.0, cE = br ? 0.0 : 2.0;
         double* red = h->red + 4 * (int64_t)i;
+        double rr[4];
+        auto read_back = [&]() -> int {
+            PURIFY_CUDA_TRY(cudaMemcpyAsync(rr, red, sizeof(rr), cudaMemcpyDeviceToHost, s));
+            PURIFY_CUDA_TRY(cudaStreamSynchronize(s));
+            return PURIFY_OK;
+        };
         int r;
         if (mixed) {
             MixedState* ms = h->mixed;
@@ -647,25 +653,26 @@ extern "C" int purify_estimate_gap(purify_t h, int lanczos_steps, double* homo_o
             st.max_ctas = ms->ctas;
             attach_products(h, &st);
             r = launch_digit_step(st, s);
+            if (r == PURIFY_OK) r = read_back();
         } else {
             const double* Xi = Xf[(i + 1) & 1];
+            r = PURIFY_OK;
             if (digits) {
                 int redo = -1;
                 r = f64d_step(*h->f64, Xi, Xi, Xi, Xf[i & 1], n, cP, cE, 0.0, 1.0, 0.0, red, s);
+                if (r == PURIFY_OK) r = f64d_read(*h->f64, s);
+                if (r == PURIFY_OK) r = read_back();
                 if (r == PURIFY_OK) r = check_f64(h, &redo);
                 if (r == PURIFY_OK && redo >= 0) digits = false;  // X_i does not fit in digits
             }
-            if (!digits) r = launch_step_f64(Xi, Xi, Xi, Xf[i & 1], n, cP, cE, 0.0, 1.0, 0.0, red, s);
+            if (r == PURIFY_OK && !digits) {
+                r = launch_step_f64(Xi, Xi, Xi, Xf[i & 1], n, cP, cE, 0.0, 1.0, 0.0, red, s);
+                if (r == PURIFY_OK) r = read_back();
+            }
         }
         if (r != PURIFY_OK) {
             release();
             return r;
-        }
-        double rr[4];
-        if (cudaMemcpyAsync(rr, red, sizeof(rr), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess) {
-            release();
-            return PURIFY_ERR_CUDA;
         }
         const double idem_in = std::sqrt(std::max(rr[1], 0.0));
         if (i > 0 && idem_in < thr && std::llround(tr_prev) == h->nocc) {

@@ -199,7 +199,8 @@ int ensure_dense_F(purify_ctx* h);
 // as for f64d_begin.  Where the size or the device's memory does not allow
 // them, f64_on stays false and the steps take the float64 FMA kernel.
 int begin_f64(purify_ctx* h, int operands);
-// f64d_check of the handle's products; a wait that ran out goes to st.device_flag.
+// f64d_check of the handle's products (after f64d_read and a synchronisation); a
+// wait that ran out goes to st.device_flag.
 int check_f64(purify_ctx* h, int* redo_from);
 // After the steps: large buffers go back to the device (f64d_end).
 void end_f64(purify_ctx* h);

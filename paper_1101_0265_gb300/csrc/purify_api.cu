@@ -381,7 +381,7 @@ int purify::begin_f64(purify_ctx* h, int operands) {
 
 int purify::check_f64(purify_ctx* h, int* redo_from) {
     int flag = 0;
-    const int r = f64d_check(*h->f64, h->stream, redo_from, &flag);
+    const int r = f64d_check(*h->f64, redo_from, &flag);
     if (flag) h->st.device_flag = flag;
     return r;
 }
@@ -880,6 +880,8 @@ static int refine_f64(purify_ctx* h, int R) {
     PURIFY_TRY(r);
     if (digits) {
         int redo = -1;
+        PURIFY_TRY(f64d_read(*h->f64, h->stream));
+        PURIFY_CUDA_TRY(cudaStreamSynchronize(h->stream));
         PURIFY_TRY(check_f64(h, &redo));
         if (redo >= 0) {  // from the refinement step that could not be finished; its input is intact
             const int r0 = redo / 2;
@@ -904,7 +906,10 @@ static int refine_f64(purify_ctx* h, int R) {
 // the test of what digits leave of the density's small entries.
 static int end_fp64_steps(purify_ctx* h, size_t doubles, std::vector<double>& red_host) {
     PURIFY_CUDA_TRY(cudaEventRecord(h->e1, h->stream));
-    if (h->f64_on) PURIFY_TRY(f64d_test_entries(*h->f64, h->X[h->cur], h->F, h->n, h->stream));
+    if (h->f64_on) {
+        PURIFY_TRY(f64d_test_entries(*h->f64, h->X[h->cur], h->F, h->n, h->stream));
+        PURIFY_TRY(f64d_read(*h->f64, h->stream));
+    }
     red_host.assign(doubles, 0.0);
     PURIFY_CUDA_TRY(cudaMemcpyAsync(red_host.data(), h->red, sizeof(double) * red_host.size(), cudaMemcpyDeviceToHost,
                                     h->stream));

@@ -36,6 +36,8 @@ cudaError_t cudaFree(void* p) {
     free(p);
     return cudaSuccess;
 }
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return cudaMalloc(p, n); }
+cudaError_t cudaFreeHost(void* p) { return cudaFree(p); }
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) {
     memset(p, v, n);
     if (n > 64) {  // the sums (the flags are two ints)
@@ -99,7 +101,8 @@ static bool begin() {
 static int step() { return f64d_step(f, X, X, X, X + 1, 200, 1.0, 0.0, 0.0, 1.0, 0.0, red, nullptr); }
 static int check() {
     int redo = 0, flag = 0;
-    return f64d_check(f, nullptr, &redo, &flag);
+    const int r = f64d_read(f, nullptr);
+    return r == PURIFY_OK ? f64d_check(f, &redo, &flag) : r;
 }
 // The finish pass of a step that ends well clears the sums it has read.
 static int good_step_and_check() {
@@ -146,7 +149,8 @@ int main() {
     CHECK(step() == PURIFY_OK);
     f.flags[0] = 1;
     int redo = -1, flag = 0;
-    CHECK(f64d_check(f, nullptr, &redo, &flag) == PURIFY_OK && redo == 0);
+    CHECK(f64d_check(f, &redo, &flag) == PURIFY_ERR_INTERNAL);  // (not read back yet)
+    CHECK(f64d_read(f, nullptr) == PURIFY_OK && f64d_check(f, &redo, &flag) == PURIFY_OK && redo == 0);
     CHECK(begin() && sums_are_zero());
     f64d_free(f);
     printf(g_bad ? "failed\n" : "ok\n");
