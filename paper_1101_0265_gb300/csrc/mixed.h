@@ -71,7 +71,7 @@ struct MixedState {
     const double* tg_red = nullptr;
     const double* tg_D = nullptr;
     const void* tg_X0 = nullptr;
-    int tg_fixed = 0;
+    int tg_fixed = 0, tg_products = 0;
     // a whole run as queue launches: staging (host and device copies)
     std::vector<uint8_t> qhost;
     void* qdev = nullptr;

@@ -17,6 +17,7 @@
 #include <mutex>
 
 #include "digits_tc.h"
+#include "digits_fixed.h"
 #include "mixed.h"
 
 namespace purify {
@@ -191,7 +192,7 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
         PURIFY_TRY(prepare_digit_kernels());
         cudaGraph_t g = nullptr;
         PURIFY_CUDA_TRY(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-        int rc = PURIFY_OK;
+        int rc = PURIFY_OK, products = 0;  // product kernels of a block (two launches each on the path of small ones)
         for (int j = 0; j < kBlock && rc == PURIFY_OK; ++j) {
             trace_sched_kernel<<<1, 32, 0, h->stream>>>(dev, red, trF, j, kBlock, 0);
             for (int s = smin; s <= smax && rc == PURIFY_OK; ++s) {
@@ -215,10 +216,12 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
                 attach_products(h, &st);
                 tuned_shape_if_known(h->device, &st);
                 rc = launch_digit_step(st, h->stream);
+                products += digits_fixed_wanted(st) ? 2 : 1;
             }
         }
         if (rc == PURIFY_OK) trace_sched_kernel<<<1, 32, 0, h->stream>>>(dev, red, trF, kBlock, kBlock, 1);
         const cudaError_t ce = cudaStreamEndCapture(h->stream, &g);
+        count_launches(-products);  // captured, not launched
         if (rc != PURIFY_OK) {
             if (g) cudaGraphDestroy(g);
             return rc;
@@ -235,6 +238,7 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
         ms->tg_D = h->X[0];
         ms->tg_X0 = ms->Xd[0];
         ms->tg_fixed = fixed_gen;
+        ms->tg_products = products;
         ms->tg_wait = o.wait_kcycles;
         ms->tg_split = o.split_k;
     }
@@ -280,7 +284,7 @@ int run_mixed_trace_graph(purify_ctx* h, int scheme, double tol, int max_iter, S
     h->st.digit_max = dmax;
     h->st.tensor_flops = tflops;
     h->st.product_launches = m;
-    count_launches(blocks * (kBlock * (1 + smax - smin + 1) + 1) + 2);
+    count_launches(blocks * (ms->tg_products + kBlock + 1));  // with the schedule's kernels
     h->st.trace = m > 0 ? h->hist_trace.back() : NAN;
     h->st.idem_err_fro = m > 0 ? h->hist_idem.back() : NAN;
     *iters = m;
