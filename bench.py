@@ -33,7 +33,7 @@ GAPS = (1e-1, 1e-2, 1e-3, 1e-4)
 SCHEMES = ("TC_SF", "FIXED_MU_SF")
 SMS = 152                        # GB300 streaming multiprocessors
 TENSOR_FLOP_PER_CLK_SM = 8192    # dense bf16 tcgen05 rate per SM and clock (nominal)
-F64_DIGIT_PAIRS = 43             # bf16 digit pairs of one float64 product (csrc/f64_digits.cu)
+FP64_FLOP_PER_CLK_SM = 4         # two float64 FMAs per SM and clock (nominal)
 # The tensor pipe's active share of one queue launch of the digit-plane
 # product (ncu sm__pipe_tensor_cycles_active of digit_gemm_kernel<32, 5, 2>:
 # one TC_SF run at n = 4096, 14 products in one launch).
@@ -514,6 +514,25 @@ def summarize_accuracy(results, bound=1e-6):
             "max_trace_err": worst("trace_err"), "max_idem_err_fro": worst("idem_err_fro")}
 
 
+def fp64_roofline(acc, pk, pk_kind, sm_mhz):
+    """The float64 path's products against the unit they ran on: digit products on the
+    tensor cores when the runs issued tensor flops, else the float64 FMA pipe."""
+    if acc["tensor_flops"] > 0.0:
+        achieved = acc["tensor_flops"] / acc["prod_s"] / 1e12
+        peak = pk["bf16_tflops_sustained"]
+        return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                "frac": achieved / peak, "traffic": None,
+                "kernel": "float64 step: split, f64_digit_product_kernel (digit products on tcgen05), finish",
+                "peak_kind": f"{pk_kind} bf16 sustained",
+                "useful_tflops_in_products": acc["useful"] / acc["prod_s"] / 1e12}
+    achieved = acc["useful"] / acc["prod_s"] / 1e12
+    peak = SMS * FP64_FLOP_PER_CLK_SM * sm_mhz * 1e6 / 1e12
+    return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            "frac": achieved / peak, "traffic": None, "kernel": "step_f64_kernel",
+            "peak_kind": f"float64 FMA pipe: {SMS} SMs x {FP64_FLOP_PER_CLK_SM // 2} DFMA per clock x 2 "
+                         f"x the median SM clock under load ({sm_mhz:.0f} MHz)"}
+
+
 def main():
     t_start = time.perf_counter()
     args = parse()
@@ -713,15 +732,7 @@ def main():
                               "rate": f"{TENSOR_FLOP_PER_CLK_SM} dense bf16 flop per clock per SM "
                                       f"x {SMS} SMs (the nominal dense rate)"}}
     else:
-        t128 = (n + 127) // 128
-        pair_flops = t128 * (t128 + 1) / 2 * 2 * 128 * 128 * t128 * 128
-        achieved = acc["mults"] * F64_DIGIT_PAIRS * pair_flops / acc["prod_s"] / 1e12
-        peak = pk["bf16_tflops_sustained"]
-        roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": achieved / peak, "traffic": None,
-                "kernel": "float64 step: split, f64_digit_product_kernel (exact digit products on tcgen05), finish",
-                "peak_kind": f"{pk_kind} bf16 sustained", "digit_pairs": F64_DIGIT_PAIRS,
-                "useful_tflops_in_products": acc["useful"] / acc["prod_s"] / 1e12}
+        roof = fp64_roofline(acc, pk, pk_kind, sm_mhz)
     line = {
         "metric": METRIC, "value": value, "unit": "matrices/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,

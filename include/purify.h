@@ -202,7 +202,8 @@ typedef struct purify_stats_t {
     double seconds;             /* device time of the iteration loop                     */
     double lmin, lmax, homo, lumo, mu;  /* landmarks used                              */
     double useful_flops;        /* n^2 (n + 1) per symmetric product                     */
-    double tensor_flops;        /* MMA flops issued on the tensor cores (MIXED)          */
+    double tensor_flops;        /* MMA flops of the products on the tensor cores (0: a
+                                   FP64 run of the FMA kernel)                           */
     int digit_max;              /* MIXED: largest digit count used                       */
     int kernel_launches;        /* kernels launched by the last set/run call             */
     int product_launches;       /* matrix-product kernels among them (last run)          */

@@ -835,6 +835,11 @@ int ensure_planes(F64Digits& f, int b) {
 
 bool f64d_wanted(int64_t n) { return n >= kF64DigitsMinN && n <= kF64DigitsMaxN; }
 
+double f64d_flops(int64_t n) {
+    const double T = pad128(n) / TILE;
+    return 43.0 * (T * (T + 1) / 2) * (2.0 * TILE * TILE) * (T * TILE);  // 43 digit pairs
+}
+
 bool f64d_begin(F64Digits& f, int64_t n, int operands, long long wait_cycles, cudaStream_t s, int* err) {
     *err = PURIFY_OK;
     if (!f64d_wanted(n)) return false;

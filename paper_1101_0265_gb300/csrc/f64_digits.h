@@ -35,6 +35,9 @@ bool f64d_wanted(int64_t n);
 // receives other failures.
 bool f64d_begin(F64Digits& f, int64_t n, int operands, long long wait_cycles, cudaStream_t s, int* err);
 
+// MMA flops of one step's product.
+double f64d_flops(int64_t n);
+
 // launch_step_f64 by exact digit products (red[2] is not reduced); A, B and E are
 // exactly symmetric.
 int f64d_step(F64Digits& f, const double* A, const double* B, const double* E, double* C, int64_t n, double cP,

@@ -831,10 +831,12 @@ static int step64(purify_ctx* h, const double* A, const double* B, const double*
                   double cP, double cE, double cI, double dY, double dI, int64_t slot) {
     PURIFY_TRY(product_begin(h));
     double* red = h->red + 4 * slot;
-    if (h->f64_on)
+    if (h->f64_on) {
         PURIFY_TRY(f64d_step(*h->f64, A, B, E, C, h->n, cP, cE, cI, dY, dI, red, h->stream));
-    else
+        h->st.tensor_flops += f64d_flops(h->n);
+    } else {
         PURIFY_TRY(launch_step_f64(A, B, E, C, h->n, cP, cE, cI, dY, dI, red, h->stream));
+    }
     ++h->st.product_launches;
     return product_end(h);
 }
@@ -1108,6 +1110,7 @@ static int run_fp64(purify_ctx* h, int scheme, double tol, int max_iter, double 
         }
         h->pev_used = 0;
         h->st.product_launches = 0;
+        h->st.tensor_flops = 0.0;
     }
     return run_fp64_steps(h, scheme, tol, max_iter, mu, S, trace_rule, iters_out, red_host);
 }

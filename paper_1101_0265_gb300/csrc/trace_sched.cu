@@ -16,8 +16,8 @@
 #include <cstring>
 #include <mutex>
 
-#include "digits_tc.h"
 #include "digits_fixed.h"
+#include "digits_tc.h"
 #include "mixed.h"
 
 namespace purify {
