@@ -80,13 +80,13 @@ extern "C" {
 
 /* ---- arithmetic of the matrix products -------------------------------- */
 #define PURIFY_FP64    0  /* float64: products from 8 integer digit planes per operand on
-                             the tensor cores (an entry is known to about 2^-57 of its
-                             rows' 2-norms), or float64 FMA on the SIMT pipe: for small n
-                             (< 160), n above 32768, values the digits cannot hold
-                             (infinities, NaN, row scales above 2^400), too little device
-                             memory, and densities with entries so far below their rows'
-                             norms (decaying or weakly coupled matrices) that FMA
-                             knows them better                                       */
+                             the tensor cores (an entry is off by about 2^-57 of its two
+                             rows' 2-norms, at worst 4 sqrt(n) times that), or float64
+                             FMA on the SIMT pipe: for small n (< 160), n above 32768,
+                             values the digits cannot hold (infinities, NaN, row scales
+                             above 2^400), too little device memory, and densities with
+                             entries so far below their rows' norms (decaying or weakly
+                             coupled matrices) that FMA knows them better            */
 #define PURIFY_MIXED   1  /* float64 values held as integer digit planes in bf16,
                              multiplied exactly on the tcgen05 tensor cores with
                              fp32 accumulation in tensor memory, recombined in

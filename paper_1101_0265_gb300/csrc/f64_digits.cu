@@ -2,11 +2,12 @@
 //
 // GB300's float64 pipe runs 2 FMAs per clock and SM (1.26 TFLOP/s on the
 // chip), so a float64 product there is bound by that pipe at any size.  Here
-// the product is taken on the bf16 tensor pipe (1.9 PFLOP/s measured) without
-// giving up float64 accuracy: the operands are cut into integer digits whose
-// products and sums are exact in the fp32 accumulators, and the sums are put
-// together in 64-bit integers (the error-free splitting of Ozaki, Ogita,
-// Oishi and Rump, Numer. Algorithms 59 (2012), with digits of 7 bits).
+// the product is taken on the bf16 tensor pipe (1.9 PFLOP/s measured) with
+// float64's accuracy relative to the rows' norms: the operands are cut into
+// integer digits whose products and leading sums are exact in the fp32
+// accumulators, and the sums are put together in 64-bit integers (the error-free
+// splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59 (2012), with
+// digits of 7 bits).
 //
 // Digits.  Row i of a symmetric operand has the exponent e_i with
 // ||x_i||_2 <= 2^e_i (and > 2^(e_i - 2)); x_ij = 2^(e_i - 8) sum_p d_p 2^(-7p)
@@ -17,18 +18,20 @@
 // Product.  P_ij = 2^(e_i + e_j - 16) sum_l 2^(-7l) L_l with the level sums
 // L_l = sum_{p + q = l} sum_k d_p(i, k) d_q(j, k), l = 0..8 (p, q <= 7): 43
 // digit pairs.  What is left out (levels >= 9 and the digits' own rounding) is
-// about 2^-58 of ||x_i|| ||x_j||, below the rounding of a chain of n float64
-// FMAs.  (Without level 8, 36 pairs, off-diagonal entries came out 2.5 times
-// further off than with FMAs at n = 4096.)  A level sum over at most 1024 columns stays below 2^24 for
-// l <= 4 whatever the digits are (Cauchy-Schwarz for the pairs with d_0, at
-// most 3 x 1024 x 2^12 for the others) and is then exact in fp32; level 5 may
-// exceed it by a sixteenth in the worst case, at 2^-51 of the leading term per
-// unit, and levels 6 to 8 need no exactness.  So an accumulator is emptied at
-// least every 1024 columns, as an integer: each segment adds its levels,
-// shifted into units of 2^(e_i + e_j - 60), to a 64-bit integer per element
-// (|P_ij| <= 2^(e_i + e_j): the sum fits).  Integer sums do not depend on
-// their order, so the k-range of a tile may be cut anywhere and the result is
-// the same on every run and for any grid.
+// about 2^-57 of ||x_i|| ||x_j|| (at worst 4 sqrt(n) times that), for dense rows
+// below the rounding of a chain of n float64 FMAs.  (With level 8 cut to its middle
+// pair, 37 pairs, off-diagonal entries came out 2.5 times further off than with
+// FMAs at n = 4096.)  A level sum over at most 1024 columns stays below 2^24 for l
+// <= 4 whatever the digits are (Cauchy-Schwarz for the pairs with d_0, at most 3 x
+// 1024 x 2^12 for the others) and is then exact in fp32; level 5 may exceed it by a
+// sixteenth in the worst case, at 2^-51 of the leading term per unit, and levels 6
+// to 8 are rounded in fp32 (7 and 8 once more, to 32 of level 7's units, when they
+// are emptied).  So an accumulator is emptied at least every 1024 columns, as an
+// integer: each segment adds its levels, shifted into units of 2^(e_i + e_j - 60),
+// to a 64-bit integer per element (|P_ij| <= 2^(e_i + e_j): the sum fits).
+// Integer sums do not depend on their order, so the result is the same on every
+// run; with another number of SMs the segments are cut elsewhere and the last
+// bits, from level 5 on, may differ.
 //
 // Work.  Eight 128 x 128 accumulators would need twice the 512 columns of
 // tensor memory, so a tile's range is done in two passes: levels 0..3 from
@@ -36,13 +39,14 @@
 // and 8 share an accumulator).
 // Whole waves of tiles go round-robin, so that the CTAs walk k together and
 // share panels in L2; the tiles of the last, partial wave are cut evenly over
-// the grid at stage boundaries (at n = 256, three tiles on 103 CTAs).
+// the grid at stage boundaries (at n = 256, three tiles on 72 of 103 CTAs).
 //
 // Measured, one step (float64 FMA kernel -> here): n = 256 23 -> 19 us, n = 1000
 // 896 -> 57 us, n = 4096 56 ms -> 1.69 ms, of which the product kernel is about 1.5
-// ms: 2.0 PFLOP/s of digit pairs (cuBLAS bf16 burst: 1.9).  Errors of
-// one step against extended precision at n = 4096: largest 2.2e-15 -> 7e-17,
-// rms 1.8e-17 -> 2.4e-18.
+// ms: 2.0 PFLOP/s of digit pairs (cuBLAS bf16 burst: 1.9).  Errors of one step on
+// a dense rotated matrix against extended precision at n = 4096: largest 2.2e-15
+// -> 7e-17, rms 1.8e-17 -> 2.4e-18.  Matrices with entries far below their rows'
+// norms are another matter: see the test of the result below.
 //
 // A step is three launches: split (unless the operand's digits are still at
 // hand), product, finish.  An operand with an infinity, a NaN or a row scale
@@ -83,9 +87,11 @@ constexpr int kHiCost = 20, kLoCost = 33;
 constexpr int kRange32 = 32;  // 1024 columns between two emptyings, in 32-column chunks
 constexpr int kCost32 = kHiCost + 2 * kLoCost;
 constexpr int kRangeCost = kRange32 * kCost32;
-// A CTA gets at least this much of the last wave: one stage, so that in small
-// products no CTA empties its accumulators twice (n = 256, per step: 20.5 us with
-// 20, 24.6 with 30, 25.0 with 60; from n = 333 on the grid is full and it does not matter)
+// A CTA's share of the last wave is at least this: one high stage, so that in small
+// products no CTA empties its accumulators twice. (A low stage costs 33, so some
+// shares hold the start of no stage: 31 of 103 at n = 256.) n = 256, per step: 20.5
+// us with 20, 24.6 with 30, 25.0 with 60; from n = 333 on the grid is full and it
+// does not matter.
 constexpr int kMinCost = 20;
 constexpr int ERR_F64_WAIT = 32;
 constexpr int kSmemBytes = 1024 + kStages * kStageBytes + 256;
@@ -707,19 +713,21 @@ f64_finish_kernel(uint2* __restrict__ T, const int* __restrict__ ea, const int* 
 //
 // A chain of FMAs keeps P_ij to about n 2^-53 S_ij with S_ij = sum_k |x_ik| |x_kj|;
 // digits keep it to about 2^-57 ||x_i|| ||x_j||, which is no worse while S_ij >=
-// ||x_i|| ||x_j|| / (16 n).  Dense iterates are far above that (rotated spectra of
-// fillings 0.25 to 0.7: 40 to 500 times, n = 160 to 1000), but in a matrix that
+// ||x_i|| ||x_j|| / (16 n).  Dense densities are far above that (rotated spectra of
+// fillings 0.25 to 0.7: 330 to 6800 times, n = 160 to 1000), but in a matrix that
 // decays away from the diagonal, or whose parts are weakly coupled, the entries
 // between distant rows are far below it (gapped alternating chain, n = 240:
-// relative errors of 1e-7 at entries of 3e-12, nothing left below 1e-18).  So the density of a run is
-// tested pair by pair, and a run with a pair below the bound is the FMA kernel's.
-// The iterates need no test of their own: where one of them has small entries and
-// the density has none, those do not show in it beyond 2^-57 of the norms.
-
-// Both kernels are bound by reading D at large n and by latency at small n. They
-// work in float32 and go to float64 only for what does not fit there: all in
-// float64 they took 36 us of a call at n = 1000 and 230 us at n = 4096 (1.6 and 24.6
-// ms), now 12 and 140 us (n = 256: nothing that shows).
+// relative errors of 1e-7 at entries of 3e-12, nothing left below 1e-18).  So the
+// density of a run is tested pair by pair, and a run with a pair below the bound
+// is the FMA kernel's.  The iterates need no test of their own: where one of them
+// has small entries and the density has none, those do not show in it beyond
+// 2^-57 of the norms.
+//
+// Both kernels work in float32 and go to float64 only for what does not fit there;
+// the conversions still fill the float64 pipe (row pass at n = 4096: 43 us, that
+// pipe 90 % busy; reading D takes 20). All in float64 the test was 36 us of a call
+// at n = 1000 and 230 us at n = 4096 (1.6 and 24.6 ms), now 12 and 140 us (n = 256:
+// nothing that shows).
 
 struct RowScale {
     double inv;      // 1 / ||d_i|| (0: the row is below 2^-400 and not tested)
@@ -993,7 +1001,7 @@ void f64d_free(F64Digits& f) {
     }
     cudaFree(f.T);
     cudaFree(f.flags);
-    cudaFreeHost(f.host_flags);
+    if (f.host_flags) cudaFreeHost(f.host_flags);
     cudaFree(f.rows);
     f = F64Digits();
 }
