@@ -460,7 +460,7 @@ int purify_batch_get_density(purify_batch_t b, int id, double* D, int64_t ld);
 int purify_batch_stats(purify_batch_t b, int id, purify_stats_t* st);
 
 /* Free an instance's device memory (its id stays invalid afterwards), in the
- * order of the batch's stream; the batch keeps at most 2 GB of freed memory for
+ * order of the batch's stream; the batch keeps at most 8 GB of freed memory for
  * the instances added next. */
 int purify_batch_release(purify_batch_t b, int id);
 

@@ -100,21 +100,14 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // An instance's buffers are one allocation from the batch's own memory pool:
 // six cudaMalloc and cudaFree per instance, each of which waits for the device,
 // took 13 of the 22 ms of a 48-instance batch (n in [64, 2048]) from add to
-// release.  That batch takes 0.7 GiB, ten requests of up to n = 4096 1.4 GiB.  Freed
-// memory beyond kPoolKeep goes back to the device when an instance is released,
-// all of it when an allocation fails or the batch is destroyed.
-constexpr uint64_t kPoolKeep = 2ull << 30;
+// release.  Freed memory beyond kPoolKeep goes back to the device at the next
+// synchronisation, all of it when an allocation fails or the batch is destroyed.
+constexpr uint64_t kPoolKeep = 8ull << 30;
 
-// The threshold counts what instances hold too: it follows bytes_in_use.  Where the
-// pool holds more (after a release), it is trimmed at once: other allocations of
-// the process cannot have what it keeps.
+// The threshold counts what instances hold too: it follows bytes_in_use.
 int pool_threshold(purify_batch* B) {
-    uint64_t keep = kPoolKeep + B->bytes_in_use, held = 0;
+    uint64_t keep = kPoolKeep + B->bytes_in_use;
     PURIFY_CUDA_TRY(cudaMemPoolSetAttribute(B->pool, cudaMemPoolAttrReleaseThreshold, &keep));
-    PURIFY_CUDA_TRY(cudaMemPoolGetAttribute(B->pool, cudaMemPoolAttrReservedMemCurrent, &held));
-    if (held <= keep) return PURIFY_OK;
-    PURIFY_CUDA_TRY(cudaStreamSynchronize(B->stream));
-    PURIFY_CUDA_TRY(cudaMemPoolTrimTo(B->pool, keep));
     return PURIFY_OK;
 }
 
@@ -646,10 +639,10 @@ int purify_batch_add(purify_batch_t B, const double* F, int64_t n, int64_t ld, i
     }
     plan_steps(B, *in);
     in->id = (int)B->inst.size();
-    *id = in->id;
     B->inst.push_back(in);
     B->bytes_in_use += in->bytes;
     PURIFY_TRY(pool_threshold(B));
+    *id = in->id;
     return join_streams(B->user_stream, B->stream, B->join_ev);
 }
 
@@ -933,12 +926,13 @@ int purify_batch_release(purify_batch_t B, int id) {
     free_instance(B, *in);
     delete in;
     B->inst[id] = nullptr;
+    PURIFY_TRY(pool_threshold(B));
     if (B->graph) {
         cudaGraphExecDestroy(B->graph);
         B->graph = nullptr;
         B->graph_ids.clear();
     }
-    return pool_threshold(B);
+    return PURIFY_OK;
 }
 
 int64_t purify_batch_bytes_in_use(purify_batch_t B) { return B ? (int64_t)B->bytes_in_use : 0; }
