@@ -78,3 +78,25 @@ def test_large_float64_workspaces_are_given_back(P):
         held = before - _free()
     # F, two iterates and the product buffer; digits and sums of this size (1.3 GiB) are given back
     assert held <= 4 * 8 * n * n + 64 * MiB, held / MiB
+
+
+def test_rounds_of_a_batch_do_not_add_up(P):
+    n = 8192
+    F, h = I.reflected_hamiltonian_device(I.InstanceSpec(n=n, nocc=n // 2, gap=0.1, scheme="TC_SF", instance=1, config=112))
+    B = P.Batch()
+    before = _free()
+
+    def add():
+        return [B.add(F, h.nocc, h.lmin, h.lmax, h.homo, h.lumo, scheme="TC_SF", tol=1e-9, mu=0.0) for _ in range(2)]
+
+    ids = add()
+    most = before - _free()
+    assert most >= B.bytes_in_use()
+    for _ in range(3):
+        for i in ids:
+            B.release(i)
+        assert B.bytes_in_use() == 0 and before - _free() <= most
+        ids = add()
+        assert before - _free() <= most + 64 * MiB
+    B.close()
+    assert before - _free() <= 64 * MiB
