@@ -16,11 +16,10 @@
 // the order in which a finish adds the parts are those of the persistent
 // kernel, so the densities are the same bit for bit.
 //
-// A leading level that is not finite or out of any iterate's range (2^22: a
-// product's entry of 64 where iterates stay below 1; a quarter of it in a tile's
-// part, so that the sum of four fits) poisons the run: the finish pass writes NaN
-// from then on, and the caller runs it again on the persistent kernel, which
-// carries such values.
+// A leading level that is not finite or out of any iterate's range (2^20: a
+// product's entry of 16 where iterates stay below 1; the sum of a tile's four
+// parts still fits) poisons the run: the finish pass writes NaN from then on, and
+// the caller runs it again on the persistent kernel, which carries such values.
 //
 // Measured per product of a run, host calls included (persistent kernel -> here):
 // n = 200 67 -> 17 us, n = 1101 92 -> 38 us, n = 2000 at 5 digits 130 -> 110 us, n =
@@ -252,7 +251,6 @@ __global__ void __maxnreg__(kMaxRegs) digit_fixed_kernel(const __grid_constant__
             // column-major inside a tile: a warp writes 32 consecutive values
             const int off = quarter * 32 + lane + col0 * TILE;
             const bool part = t >= L.split_begin;
-            const float most = part ? 1048576.f : 4194304.f;
             unsigned long long* sum =
                 (part ? L.sums.parts + (size_t)((t - L.split_begin) / L.ways) * (TILE * TILE)
                       : L.sums.levels + (size_t)t * (TILE * TILE)) + off;
@@ -277,7 +275,7 @@ __global__ void __maxnreg__(kMaxRegs) digit_fixed_kernel(const __grid_constant__
                 for (int c = 0; c < 8; ++c) {
                     if (exact) {
                         const float a0 = __uint_as_float(v[c]), a1 = __uint_as_float(v[8 + c]);
-                        bad |= !(fabsf(a0) < most) || (NA > 1 && !(fabsf(a1) < 32768.f));
+                        bad |= !(fabsf(a0) < 1048576.f) || (NA > 1 && !(fabsf(a1) < 32768.f));
                         const unsigned long long x = pack_levels<NA>(a0, a1, __uint_as_float(v[16 + c]));
                         if (part)
                             atomicAdd(sum + (8 * q + c) * TILE, x);
