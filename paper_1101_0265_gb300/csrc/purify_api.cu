@@ -888,6 +888,7 @@ static int refine_f64(purify_ctx* h, int R) {
         if (redo >= 0) {  // from the refinement step that could not be finished; its input is intact
             const int r0 = redo / 2;
             x = h->cur ^ (r0 & 1);
+            h->st.tensor_flops -= (2 * R - redo) * f64d_flops(h->n);  // (steps that left at once)
             PURIFY_CUDA_TRY(cudaMemsetAsync(h->red + 8 * r0, 0, sizeof(double) * 8 * (R - r0), h->stream));
             PURIFY_TRY(steps(r0));
         }

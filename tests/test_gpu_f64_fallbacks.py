@@ -33,7 +33,7 @@ def _ones_run(P, n, iters, refine):
 # has an operand that they cannot hold and is made again.
 @pytest.mark.parametrize("n", [200, 300])
 def test_refinement_goes_on_with_the_fma_kernel(P, n):
-    X, _ = _ones_run(P, n, 4, 0)
+    X, st0 = _ones_run(P, n, 4, 0)
     scale = float(X.abs().max()) * n ** 0.5
     assert 2.0 ** 70 < scale < 2.0 ** 130
     D, st = _ones_run(P, n, 4, 2)
@@ -45,6 +45,9 @@ def test_refinement_goes_on_with_the_fma_kernel(P, n):
     # entries of one sign: products are exact to n 2^-53 relative, twice cubed
     assert bool(torch.isfinite(X).all()) and float((D / X - 1.0).abs().max()) <= 20 * n * 2.0 ** -53
     assert st["refine_multiplications"] == 4
+    # three of the four products were made of digits: 43 pairs each
+    t = (n + 127) // 128
+    assert st["tensor_flops"] - st0["tensor_flops"] == 3 * 43 * (t * (t + 1) // 2) * 2.0 * 128 * 128 * 128 * t
 
 
 def test_gap_estimate_of_a_diverging_iterate(P):
